@@ -83,20 +83,37 @@ __device__ __forceinline__ void rtn_grid_of(float mn, float mx, RtnGrid grid, fl
     zero = (float)rint(-xmin / (double)scale);
   }
 }
-// Running minima and maxima of two interleaved halves of the weights (NaNs are passed over, as by fminf / fmaxf).
+// Running minima and maxima of two interleaved halves of the weights.  The minimum passes NaNs over, as fminf does; the
+// maximum keeps them, so that a group with one is known (rtn_finite) at no instruction per weight.
 __device__ __forceinline__ void rtn_minmax8(const uint4& v, __half2& mn, __half2& mx) {
   const __half2* h = reinterpret_cast<const __half2*>(&v);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) { mn = __hmin2(mn, h[k]); mx = __hmax2(mx, h[k]); }
+  for (int k = 0; k < 4; ++k) { mn = __hmin2(mn, h[k]); mx = __hmax2_nan(mx, h[k]); }
 }
 __device__ __forceinline__ __half2 rtn_half2_const(unsigned short bits) { return __halves2half2(__ushort_as_half(bits), __ushort_as_half(bits)); }
 __device__ __forceinline__ float rtn_low(__half2 m) { return fminf(__low2float(m), __high2float(m)); }
-__device__ __forceinline__ float rtn_high(__half2 m) { return fmaxf(__low2float(m), __high2float(m)); }
+__device__ __forceinline__ float rtn_high(__half2 m) {      // NaN if either half is
+  const float a = __low2float(m), b = __high2float(m);
+  return isnan(a) ? a : isnan(b) ? b : fmaxf(a, b);
+}
+// True if every weight of a group with these (kept) minimum and maximum is finite.
+__device__ __forceinline__ bool rtn_finite(float mn, float mx) { return isfinite(mx) && isfinite(mn); }
+// The maximum of pieces first, first + step, ... with NaNs passed over: for a group whose kept maximum is one.
+__device__ __noinline__ float rtn_high_of_numbers(const uint4* p, int first, int pieces, int step) {
+  float mx = -INFINITY;
+#pragma unroll 1
+  for (int i = first; i < pieces; i += step) {
+    const uint4 v = __ldg(p + i);
+    const __half2* h = reinterpret_cast<const __half2*>(&v);
+    for (int k = 0; k < 4; ++k) mx = fmaxf(mx, fmaxf(__low2float(h[k]), __high2float(h[k])));
+  }
+  return mx;
+}
 template <bool kMin>
 __device__ __forceinline__ __half2 rtn_reduce_step(__half2 m, int o) {
   const uint32_t u = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<const uint32_t*>(&m), o);
   const __half2 x = *reinterpret_cast<const __half2*>(&u);
-  return kMin ? __hmin2(m, x) : __hmax2(m, x);
+  return kMin ? __hmin2(m, x) : __hmax2_nan(m, x);
 }
 // The operation the oracle performs, for the eight weights of a piece.
 template <int F>
@@ -115,8 +132,9 @@ __device__ __noinline__ uint64_t rtn_codes8_by_division(uint4 v, float scale, fl
 // added to 1.5 * 2^I: the float then holds it in fixed point, S = 23 - I fraction bits below the integer, which a shift and
 // one add-clamp turn into the code.  I leaves room for the code's range (a weight lies inside its own group's minimum and
 // maximum).  The reciprocal's and the sum's rounding are below one unit 2^-S; wherever the fraction bits are within that of
-// a tie (the constant is one unit high, so bits 0 .. 2), or the value is not finite (all fraction bits zero), the eight
-// weights go through the division.
+// a tie (the constant is one unit high, so bits 0 .. 2) the eight weights go through the division.  So do all weights of a
+// group with a NaN or an infinity in it, whose fixed-point values mean nothing (a NaN is 0x7FFFFFFF, which looks like a
+// fraction far from a tie): the caller passes rs = 0 for such a group.
 template <int F> constexpr int kRtnInt = F == 2 ? 4 : F == 3 ? 5 : F == 4 ? 6 : 10;
 template <int F>
 __device__ __forceinline__ uint64_t rtn_codes8(const uint4& v, float scale, float rs, float zero, int maxq) {
@@ -125,7 +143,7 @@ __device__ __forceinline__ uint64_t rtn_codes8(const uint4& v, float scale, floa
   constexpr int kBias = (0x3F800000 + (kRtnInt<F> << 23) + 0x400000) >> S;     // upper bits of kBig
   const __half2* h = reinterpret_cast<const __half2*>(&v);
   const float base = zero + (kBig + 0.5f + 1.f / (float)(1 << S));
-  uint32_t word[2] = {0u, 0u}, frac = 0xFFFFFFFFu;
+  uint32_t word[2] = {0u, 0u}, frac = rs > 0.f ? 0xFFFFFFFFu : 0u;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const float2 w2 = __half22float2(h[k >> 1]);
@@ -177,14 +195,20 @@ rtn_fused_kernel(const __half* __restrict__ W, int R, int C, int g, int G, RtnGr
   }
   for (; i0 < pieces; i0 += 32) { const uint4 a = __ldg(p + i0); rtn_minmax8(a, mn, mx); }
   for (int o = 16; o > 0; o >>= 1) { mn = rtn_reduce_step<true>(mn, o); mx = rtn_reduce_step<false>(mx, o); }
+  float lo = rtn_low(mn), hi = rtn_high(mx);                // (the same in every lane)
+  const bool finite = rtn_finite(lo, hi);
+  if (isnan(hi)) {
+    hi = rtn_high_of_numbers(p, lane, pieces, 32);
+    for (int o = 16; o > 0; o >>= 1) hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
   float scale = 0.f, zero = 0.f;
   if (lane == 0) {
-    rtn_grid_of(rtn_low(mn), rtn_high(mx), grid, scale, zero);
+    rtn_grid_of(lo, hi, grid, scale, zero);
     scales[wid] = scale; zeros[wid] = zero;
   }
   scale = __shfl_sync(0xffffffffu, scale, 0);
   zero = __shfl_sync(0xffffffffu, zero, 0);
-  const float rs = 1.0f / scale;
+  const float rs = finite ? 1.0f / scale : 0.f;
   // words of this group inside the row: the group starts at bit gi * g * F, a multiple of 32 F bits
   uint32_t* qrow = qweight + (int64_t)row * (C / 32 * F) + (int64_t)gi * (g / 32 * F);
   int base = 0;
@@ -242,12 +266,14 @@ rtn_span_kernel(const __half* __restrict__ W, int R, int C, int G, RtnGrid grid,
   }
   float my_scale = 1.f, my_zero = 0.f;
   const int my_group = run * 32 + lane;
+  const bool finite = rtn_finite(my_mn, my_mx);
   if (my_group < G) {
+    if (isnan(my_mx)) my_mx = rtn_high_of_numbers(p, my_group * kLanes, (my_group + 1) * kLanes, 1);
     rtn_grid_of(my_mn, my_mx, grid, my_scale, my_zero);
     scales[(int64_t)row * G + my_group] = my_scale;
     zeros[(int64_t)row * G + my_group] = my_zero;
   }
-  const float my_rs = 1.0f / my_scale;
+  const float my_rs = finite ? 1.0f / my_scale : 0.f;
   uint32_t* qrow = qweight + (int64_t)row * (C / 32 * F);
 #pragma unroll 1
   for (int sp = 0; sp < kLanes; ++sp) {

@@ -889,6 +889,39 @@ def test_rtn_fixed_point_codes_at_the_edges(B, bits, C, group, sym, scale_fp16):
     assert np.array_equal(s * (codes - z), what_ref)
 
 
+@pytest.mark.parametrize("bits", [2, 3, 4, 8, O.BITS_TERNARY])
+@pytest.mark.parametrize("C,group", [(1056, 0), (1024, 512), (288, 96), (1024, 256), (256, 64), (64, 32), (64, 8)])
+@pytest.mark.parametrize("sym,scale_fp16", [(False, False), (True, False), (False, True)])
+def test_rtn_codes_of_weights_that_are_not_numbers(B, bits, C, group, sym, scale_fp16):
+    """A NaN weight: code 0 and no say in its group's grid, whatever the group's size.  An infinite weight: an infinite scale, on which
+    it has code 0 too and every number the zero-point's (0 where that is no number)."""
+    rng = np.random.default_rng(5)
+    W = (0.02 * rng.standard_normal((9, C))).astype(np.float16)
+    bad = np.zeros((9, C), dtype=bool)
+    bad[0, 3], bad[1, 8:16], bad[2, ::5], bad[3, :], bad[4, -1] = True, True, True, True, True
+    plain = np.where(bad, np.float16(0), W)                  # (0 lies inside every grid: the grid is that of the numbers)
+    codes_ref, _ = O.rtn(plain, bits, group, sym, scale_fp16=scale_fp16)
+    g = group if group > 0 else C
+    W = np.where(bad, np.float16(np.nan), W)
+    inf = np.zeros((9, C // g), dtype=bool)                   # groups with an infinity
+    for r, c, v in ((6, 5, np.inf), (7, 9, -np.inf), (8, 0, np.inf), (8, C - 1, -np.inf)):
+        W[r, c] = v
+        inf[r, c // g] = True
+    W[6, 16:24] = np.inf
+    inf[6, 16 // g:(23 // g) + 1] = True
+    out = B.gptq_rtn_layer(torch.from_numpy(W).cuda(), bits, group, sym, scale_fp16=scale_fp16)
+    codes = O.unpack_codes(out["qweight"].cpu().numpy().view(np.uint32), bits, C)
+    scales, zeros = out["scales"].cpu().numpy(), out["zeros"].cpu().numpy()
+    of_inf = inf.repeat(g, 1)
+    assert np.array_equal(codes[~of_inf], np.where(bad, 0, codes_ref)[~of_inf])
+    clean = B.gptq_rtn_layer(torch.from_numpy(plain).cuda(), bits, group, sym, scale_fp16=scale_fp16)
+    for k, v in (("scales", scales), ("zeros", zeros)):
+        assert np.array_equal(v[~inf], clean[k].cpu().numpy()[~inf])
+    assert np.isposinf(scales[inf]).all()
+    z = np.nan_to_num(zeros).repeat(g, 1)                     # a number's quotient is 0 on such a scale
+    assert np.array_equal(codes[of_inf], np.where(np.isfinite(W), z, 0)[of_inf].astype(codes.dtype))
+
+
 @pytest.mark.parametrize("C", [32, 64, 96, 160, 1056])
 def test_symmetrize_at_tile_edges(B, C):
     """H[i][j] = H[j][i] below the diagonal, the rest untouched, for widths that end inside a 64-column tile."""
