@@ -217,14 +217,6 @@ __device__ __forceinline__ bool run_task(const Args& a, Smem& s, const Task& k, 
 }
 
 // ---- factor + inverse of one 64 x 64 tile (fp64) ----------------------------------------------------------
-// 1 / sqrt(d) from the hardware's approximation and one third-order step of the binomial series of (1 - e)^(-1/2),
-// e = 1 - d y^2: the error goes from e to about e^3, below fp64's last bit.
-__device__ __forceinline__ double inv_sqrt(double d) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-(d * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
 // c += a (8 x 4, row) * b (4 x 8, col): lane holds a[lane / 4][lane % 4], b[lane % 4][lane / 4], c[lane / 4][2 (lane % 4) + {0, 1}]
 __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
@@ -234,7 +226,7 @@ __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
 // last to first: x[i] = D[i][j] / sqrt(pivot) is T[i][j] for i < j and, because a row restarts from zero when its own column
 // comes, V[j][i] for i >= j; then D[i][c] -= x[i] x[c] for the earlier columns c of the eight.
 // Every lane carries the 8 x 8 diagonal block beside its own row and factors it redundantly: pivots and multipliers are in
-// registers everywhere, and the chain per column is a reciprocal root, a multiplication and a multiply-add (70 cycles).
+// registers everywhere, and the chain per column is a reciprocal root, a multiplication and a multiply-add (85 cycles).
 // (With the block's rows in eight lanes and two shuffles per multiplier and pivot a column took 240 cycles, half of the whole
 // kernel's chain.  A real loop over eight columns at a time: one warp running 32 columns unrolled, 32 KB of straight code,
 // was bound by instruction fetch and took twice as long again.)
@@ -260,7 +252,7 @@ __device__ __forceinline__ void sweep8(double (*D)[LDD], int jb, int row, int k_
       if (row == 0) report_error(dev_info, GPTQ_ERR_NOT_PD, k_global + 8 * jb + j);
       d = 1.0;
     }
-    const double rp = inv_sqrt(d);
+    const double rp = rsqrt(d);
     const bool own = row == 8 * jb + j;
     double xc[8];
 #pragma unroll
