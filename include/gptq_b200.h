@@ -161,7 +161,7 @@ gptq_status_t gptq_prepare_factor(const float* H, float damp, int C, float* F,
  * memory pool owns the whole device, a latency-critical loop where an allocation would
  * stall the GPU, a process with a fixed memory budget handed out at start-up.  Such a
  * caller has no workspace to pass, so the scratch lives inside the library, in one fixed
- * array in device global memory of 2,560 bytes (the dampening and the progress words of the panel kernel).
+ * array in device global memory of 788,992 bytes (the dampening, and the progress words and fp64 tiles of the panel kernel).
  *
  *   - Limit: C <= GPTQ_PREPARE_HINV_STATIC_MAX_C (1024); a larger C returns
  *     GPTQ_ERR_UNSUPPORTED and nothing is enqueued (use gptq_prepare_hinv with a workspace).

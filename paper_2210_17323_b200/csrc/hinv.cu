@@ -244,7 +244,7 @@ __global__ void split_diag_t_kernel(const float* __restrict__ U, int C, int j0, 
 constexpr int kNB2 = 1024;   // outer panel width: contractions over everything outside it run on the tensor cores
 
 struct HinvWs {
-  double* lam; panel::Flags* flags; __half* Fhi; __half* Flo; __half* VThi; __half* VTlo; __half* TThi; __half* TTlo;
+  double* lam; panel::Flags* flags; double* pairs; __half* Fhi; __half* Flo; __half* VThi; __half* VTlo; __half* TThi; __half* TTlo;
   __half* Vhi[2]; __half* Vlo[2]; __half* TAhi; __half* TAlo;
   float* r; float* rinv; float* rs; float* rsinv; float* u; float* uinv;      // [C] each
   float* g[2]; float* ginv[2]; float* gam; float* gam2inv;                     // [kNB2] each
@@ -255,6 +255,7 @@ HinvWs carve_hinv(void* ws, int C) {
   HinvWs o;
   o.lam = w.take<double>(1);
   o.flags = w.take<panel::Flags>(1);                              // progress of the panel kernel
+  o.pairs = w.take<double>(panel::pair_doubles(C < kNB2 ? C : kNB2));    // its fp64 tiles
   const bool outer = C > kNB2;
   o.Fhi = w.take<__half>(outer ? (size_t)C * C : 0);              // scaled fp16 hi / lo of the factor as it is finalised
   o.Flo = w.take<__half>(outer ? (size_t)C * C : 0);
@@ -416,7 +417,7 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
       }
     }
     // C2: factor D and invert it in place
-    if ((st = panel::launch(D, C, wj, j0, w.flags, dev_info, device_sm_count(), s)) != GPTQ_OK) return st;
+    if ((st = panel::launch(D, C, wj, j0, w.flags, w.pairs, dev_info, device_sm_count(), s)) != GPTQ_OK) return st;
     if (!outer || j0 == 0) continue;
     __half* Vhi = w.Vhi[J & 1]; __half* Vlo = w.Vlo[J & 1];
     float* gJ = w.g[J & 1]; float* ginvJ = w.ginv[J & 1];
@@ -550,8 +551,9 @@ extern "C" gptq_status_t gptq_prepare_factor(const float* H, float damp, int C, 
 namespace gptq {
 namespace {
 constexpr int kStaticMaxC = GPTQ_PREPARE_HINV_STATIC_MAX_C;
-// workspace of gptq_prepare_hinv at C <= 1024: lambda and the progress words of the panel kernel
-constexpr size_t kStaticScratchBytes = 256 + (sizeof(panel::Flags) + kAlign - 1) / kAlign * kAlign;
+// workspace of gptq_prepare_hinv at C <= 1024: lambda, the progress words of the panel kernel and its fp64 tiles
+constexpr size_t kStaticScratchBytes = 256 + (sizeof(panel::Flags) + kAlign - 1) / kAlign * kAlign + panel::pair_doubles(kStaticMaxC) * sizeof(double);
+static_assert(kStaticScratchBytes == 788992, "the public header states this size");
 static __device__ __align__(256) unsigned char hinv_static_scratch[kStaticScratchBytes];
 constexpr int kMaxDevices = 64;
 }  // namespace

@@ -8,6 +8,9 @@
 //   factor   M[k][k] = T_kk T_kk^T, V_kk = T_kk^-1                                (fp64, one CTA)
 //   solve    M[i][k] <- M[i][k] V_kk^T                          for every i != k   (T_ik above, V_ki^T below the diagonal)
 //   update   M[i][c] -= M[i][k] T_ck^T                          for c < k and (i <= c or i >= k)     (M[k][k] := V_kk^T)
+// Two neighbouring tile columns (2 m, 2 m + 1) are factored and inverted in fp64 as one 128 x 128 block: what they exchange
+// (V of column 2 m + 1, the tile between them, V of column 2 m) is kept in fp64 beside the matrix, and only finished entries of
+// T and V are rounded to fp32.  (With fp32 products between them U was 2 to 6 times as far from 64 bits for 96 .. 128 columns.)
 //
 // What bounds it: the chain factor -> solve of the tile above -> update of the next diagonal tile -> factor.  Everything
 // else (about 1600 tile products for w = 1024) has one step's time to finish.  So the first CTA to arrive runs that chain
@@ -15,8 +18,8 @@
 // CTAs to be resident together: a product waits only for products EARLIER in the list and for chain steps, and the
 // chain, if what it waits for has not been taken by anybody, takes it itself (chain_wait).  Every wait is bounded.
 // As separate launches (one 128-wide diagonal kernel of 97 us, two small GEMMs, two more on a side stream for the
-// inverse, per 128 columns) a 1024-wide call took 1.29 ms; this form 0.24 ms (768 columns: 0.94 -> 0.19 ms).  A chain step
-// is about 14 us: 7 in the fp64 tile, 3 in the two tile products, the rest in waiting, loads and publication.
+// inverse, per 128 columns) a 1024-wide call took 1.29 ms; this form 0.254 ms (768 columns: 0.94 -> 0.195 ms), of which the
+// fp64 products of the pairs are 0.006 ms and rsqrt() 0.009.  A chain step is about 15 us.
 #pragma once
 
 namespace gptq {
@@ -28,6 +31,9 @@ constexpr int kMaxTiles = 16;        // w <= 1024
 constexpr int kThreads = 256;
 constexpr int LDF = 68;              // fp32 tile pitch (floats): 16-byte rows, eight rows on distinct bank groups
 constexpr int LDD = 68;              // fp64 tile pitch (doubles): four rows 32 bytes apart modulo 128, conflict-free fragments
+// fp64 tiles of a pair of tile columns (k, k + 1), k even: the inverse of column k + 1's diagonal tile, the tile between them, the
+// inverse of column k's.  An inverse is kept transposed, as the factorisation leaves it: entry (m, c) is V[c][m], c <= m.
+constexpr int kPairV1 = 0, kPairT = 1, kPairV0 = 2, kPairTiles = 3;
 
 // Progress of one launch, in the caller's workspace; all zero when the kernel starts.
 struct Flags {
@@ -37,19 +43,25 @@ struct Flags {
   int abort;                         // a wait ran out: everybody leaves
   int solved[kMaxTiles * kMaxTiles]; // tile (i, k) has been through step k's solve
   int updated[kMaxTiles * kMaxTiles];// updates applied to tile (i, c)
+  int paired[kMaxTiles / 2];         // the fp64 tiles of pair (2 m, 2 m + 1) are complete
 };
+// doubles of the pairs of a block of w columns
+constexpr size_t pair_doubles(int w) { return (size_t)((w + TB - 1) / TB / 2) * kPairTiles * TB * TB; }
 
 struct Args {
   float* A;                          // first element of the block inside the C x C matrix
   int64_t ld;
   int w, nt, k_global;               // width, tiles, global index of the block's first row (for reports)
   Flags* fl;
+  double* pairs;                     // pair_doubles(w)
   int* dev_info;
 };
 
 struct Smem {
-  float As[TB][LDF];
-  float Bs[TB][LDF];
+  union {
+    struct { float As[TB][LDF]; float Bs[TB][LDF]; };
+    double E[TB][LDD];
+  };
   double D[TB][LDD];
   int msg[4];
 };
@@ -164,10 +176,78 @@ __device__ __forceinline__ void load_tile_t(const Args& a, int i, int c, float (
   }
 }
 
+// ---- fp64 tiles of a pair -------------------------------------------------------------------------------
+// c += a (8 x 4, row) * b (4 x 8, col): lane holds a[lane / 4][lane % 4], b[lane % 4][lane / 4], c[lane / 4][2 (lane % 4) + {0, 1}]
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+               : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
+}
+__device__ __forceinline__ double* pair_tile(const Args& a, int k, int which) { return a.pairs + ((size_t)(k >> 1) * kPairTiles + which) * (TB * TB); }
+__device__ __forceinline__ void load_pair_tile(const double* src, double (*S)[LDD], int t) {
+  double2 v[8];
+#pragma unroll
+  for (int p = 0; p < 8; ++p) v[p] = __ldcg(reinterpret_cast<const double2*>(src) + t + kThreads * p);
+#pragma unroll
+  for (int p = 0; p < 8; ++p) { const int e = t + kThreads * p; *reinterpret_cast<double2*>(&S[e >> 5][2 * (e & 31)]) = v[p]; }
+}
+__device__ __forceinline__ void store_pair_tile(double* dst, const double (*S)[LDD], int t) {
+#pragma unroll
+  for (int p = 0; p < 8; ++p) { const int e = t + kThreads * p; reinterpret_cast<double2*>(dst)[e] = *reinterpret_cast<const double2*>(&S[e >> 5][2 * (e & 31)]); }
+}
+// A pair's tile of the inverse, all threads: V[k][k + 1] = -V_kk T[k][k + 1] V_{k+1,k+1}, transposed into tile (k + 1, k).  Warp
+// `rt` makes the eight rows 8 rt .. of each product; entries on the wrong side of a triangle are skipped or read as zero.
+__device__ __forceinline__ bool pair_inverse(const Args& a, Smem& s, int k, int t) {
+  const int rt = t >> 5, r = (t & 31) >> 2, q = t & 3;
+  if (t == 0) s.msg[3] = wait_ge(&a.fl->paired[k >> 1], 1, a) ? 1 : 0;
+  __syncthreads();                                      // (also: the previous product is done with the tiles)
+  if (!s.msg[3]) return false;
+  load_pair_tile(pair_tile(a, k, kPairT), s.E, t);
+  load_pair_tile(pair_tile(a, k, kPairV1), s.D, t);
+  __syncthreads();
+  double y[8][2];
+#pragma unroll
+  for (int ct = 0; ct < 8; ++ct) y[ct][0] = y[ct][1] = 0.0;
+#pragma unroll
+  for (int kc = 0; kc < 16; ++kc) {
+    const double x = s.E[8 * rt + r][4 * kc + q];
+#pragma unroll
+    for (int ct = kc / 2; ct < 8; ++ct) {
+      const double v = s.D[8 * ct + r][4 * kc + q];
+      dmma(y[ct], x, 4 * kc + q <= 8 * ct + r ? v : 0.0);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int ct = 0; ct < 8; ++ct) *reinterpret_cast<double2*>(&s.E[8 * rt + r][8 * ct + 2 * q]) = make_double2(y[ct][0], y[ct][1]);
+  load_pair_tile(pair_tile(a, k, kPairV0), s.D, t);
+  __syncthreads();
+#pragma unroll
+  for (int ct = 0; ct < 8; ++ct) y[ct][0] = y[ct][1] = 0.0;
+#pragma unroll 2
+  for (int kc = 2 * rt; kc < 16; ++kc) {
+    const double v = s.D[4 * kc + q][8 * rt + r], x = 4 * kc + q >= 8 * rt + r ? v : 0.0;
+#pragma unroll
+    for (int ct = 0; ct < 8; ++ct) dmma(y[ct], x, s.E[4 * kc + q][8 * ct + r]);
+  }
+  float* out = a.A + (int64_t)(TB * (k + 1)) * a.ld + TB * k + 8 * rt + r;
+#pragma unroll
+  for (int ct = 0; ct < 8; ++ct)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int c = 8 * ct + 2 * q + e;
+      if (TB * (k + 1) + c < a.w) out[(int64_t)c * a.ld] = (float)-y[ct][e];
+    }
+  __syncthreads();
+  if (t == 0) st_release(&a.fl->solved[(k + 1) * kMaxTiles + k], 1);
+  return true;
+}
+
 // One product of the list, all threads of the CTA.  False if the launch is being abandoned.
 __device__ __forceinline__ bool run_task(const Args& a, Smem& s, const Task& k, int t) {
   const int nt = a.nt, tx = t & 15, ty = t >> 4;
   Flags* fl = a.fl;
+  if (k.c + 1 == k.k && (k.k & 1) && k.i == k.k) return true;                     // part of pair_inverse
+  if (k.kind == 0 && k.i == k.k + 1 && !(k.k & 1)) return pair_inverse(a, s, k.k, t);
   if (t == 0) {
     bool ok;
     if (k.kind == 0) {
@@ -183,7 +263,7 @@ __device__ __forceinline__ bool run_task(const Args& a, Smem& s, const Task& k, 
   if (!s.msg[3]) return false;
   float* out = a.A + (int64_t)(TB * k.i + ty) * a.ld + TB * k.c + tx;
   float old[4][4];
-  const bool first = k.kind == 1 && k.i >= k.k && k.i == k.k;   // a lower tile's first update: it starts as zero
+  const bool first = k.kind == 1 && k.i == k.k;         // a lower tile's first update: it starts as zero
 #pragma unroll
   for (int p = 0; p < 4; ++p)
 #pragma unroll
@@ -217,11 +297,6 @@ __device__ __forceinline__ bool run_task(const Args& a, Smem& s, const Task& k, 
 }
 
 // ---- factor + inverse of one 64 x 64 tile (fp64) ----------------------------------------------------------
-// c += a (8 x 4, row) * b (4 x 8, col): lane holds a[lane / 4][lane % 4], b[lane % 4][lane / 4], c[lane / 4][2 (lane % 4) + {0, 1}]
-__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-               : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
-}
 // Columns 8 jb .. 8 jb + 7 of the sweep over the 64 rows of D, by two warps: lane l of warp h holds row 32 h + l.  Column j,
 // last to first: x[i] = D[i][j] / sqrt(pivot) is T[i][j] for i < j and, because a row restarts from zero when its own column
 // comes, V[j][i] for i >= j; then D[i][c] -= x[i] x[c] for the earlier columns c of the eight.
@@ -309,10 +384,11 @@ __device__ __forceinline__ void factor64(Smem& s, int t, int k_global, int* dev_
 // ---- the chain ----------------------------------------------------------------------------------------------
 // All threads: waits until tiles (k, k) and (k, k + 1) have seen n updates.  If nobody has taken the entries of the list that
 // lead there (no other CTA of this launch is resident), this CTA runs them itself: entries below `limit` depend only on
-// steps that the chain has already passed.
-__device__ __forceinline__ bool chain_wait(const Args& a, Smem& s, int k, int n, int limit, int t) {
+// steps that the chain has already passed.  helped: it ran some, and the tiles in shared memory are not what they were.
+__device__ __forceinline__ bool chain_wait(const Args& a, Smem& s, int k, int n, int limit, int t, bool& helped) {
   const int* p = &a.fl->updated[k * kMaxTiles + k];
   uint64_t t0 = 0;
+  helped = false;
   for (;;) {
     // two threads look at one tile each
     bool ready = true;
@@ -342,55 +418,120 @@ __device__ __forceinline__ bool chain_wait(const Args& a, Smem& s, int k, int n,
     const int m = s.msg[0], ticket = s.msg[1];
     __syncthreads();
     if (m == 3) return false;
-    if (m == 2 && !run_task(a, s, task_of(a.nt, ticket), t)) return false;
+    if (m == 2) {
+      helped = true;
+      if (!run_task(a, s, task_of(a.nt, ticket), t)) return false;
+    }
   }
+}
+
+// Step k of an even column with a right neighbour, fp64: T[k][k + 1] = M[k][k + 1] V^T, and D = M[k][k] - T T^T.  D holds the
+// neighbour's inverse (transposed) on entry.
+__device__ __forceinline__ void pair_step(const Args& a, Smem& s, int k, int t) {
+  const int warp = t >> 5, r = (t & 31) >> 2, q = t & 3;
+  load_tile(a, k, k + 1, s.As, t);
+  load_tile(a, k, k, s.Bs, t);
+  __syncthreads();
+  double y[8][2];
+#pragma unroll
+  for (int ct = 0; ct < 8; ++ct) y[ct][0] = y[ct][1] = 0.0;
+#pragma unroll
+  for (int kc = 0; kc < 16; ++kc) {
+    const double x = (double)s.As[8 * warp + r][4 * kc + q];
+#pragma unroll
+    for (int ct = 0; ct < kc / 2 + 1; ++ct) {
+      const double v = s.D[4 * kc + q][8 * ct + r];
+      dmma(y[ct], x, 4 * kc + q >= 8 * ct + r ? v : 0.0);
+    }
+  }
+  __syncthreads();                                      // everybody has read V
+  float* out = a.A + (int64_t)(TB * k + 8 * warp + r) * a.ld + TB * (k + 1) + 2 * q;
+#pragma unroll
+  for (int ct = 0; ct < 8; ++ct) {
+    *reinterpret_cast<double2*>(&s.D[8 * warp + r][8 * ct + 2 * q]) = make_double2(y[ct][0], y[ct][1]);
+    if (TB * (k + 1) + 8 * ct + 2 * q < a.w) *reinterpret_cast<float2*>(out + 8 * ct) = make_float2((float)y[ct][0], (float)y[ct][1]);
+  }
+  __syncthreads();
+  if (t == 0) st_release(&a.fl->solved[k * kMaxTiles + k + 1], 1);
+  store_pair_tile(pair_tile(a, k, kPairT), s.D, t);
+  // The 36 8 x 8 pieces on or above the diagonal, column by column (piece e = rt + ct (ct + 1) / 2), five per warp side by side;
+  // the fifth of warps 4 .. 7 is not there (they repeat their first and drop it).
+  int ar[5], br[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const int e = warp + 8 * i < 36 ? warp + 8 * i : warp;
+    const int ct = e < 1 ? 0 : e < 3 ? 1 : e < 6 ? 2 : e < 10 ? 3 : e < 15 ? 4 : e < 21 ? 5 : e < 28 ? 6 : 7;
+    ar[i] = 8 * (e - ct * (ct + 1) / 2); br[i] = 8 * ct;
+  }
+  double z[5][2];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) z[i][0] = z[i][1] = 0.0;
+#pragma unroll 4
+  for (int kc = 0; kc < 16; ++kc)
+#pragma unroll
+    for (int i = 0; i < 5; ++i) dmma(z[i], s.D[ar[i] + r][4 * kc + q], s.D[br[i] + r][4 * kc + q]);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    if (warp + 8 * i >= 36) continue;
+    const float2 m = *reinterpret_cast<const float2*>(&s.Bs[ar[i] + r][br[i] + 2 * q]);
+    *reinterpret_cast<double2*>(&s.D[ar[i] + r][br[i] + 2 * q]) = make_double2((double)m.x - z[i][0], (double)m.y - z[i][1]);
+  }
+  __syncthreads();
 }
 
 __device__ __forceinline__ bool run_chain(const Args& a, Smem& s, int t) {
   const int nt = a.nt, tx = t & 15, ty = t >> 4;
   for (int k = nt - 1; k >= 0; --k) {
-    float old[4][4], acc[4][4];
-    const float* Mkk = a.A + (int64_t)(TB * k + ty) * a.ld + TB * k + tx;
-    auto load_diag = [&]() {
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int r = ty + 16 * p, c = tx + 16 * q;
-          old[p][q] = r == c ? 1.f : 0.f;                               // rows beyond the block: identity
-          if (TB * k + r < a.w && TB * k + c < a.w && r <= c) old[p][q] = __ldcg(Mkk + (int64_t)(16 * p) * a.ld + 16 * q);
-          acc[p][q] = 0.f;
-        }
-    };
-    if (k < nt - 1) {
-      // T[k][k + 1] = M[k][k + 1] V^T, and its update of tile (k, k).  (Bs holds V_{k+1}, left there by the last step.)
-      const int limit = tasks_before_step(nt, k + 1), n = nt - 2 - k;
-      if (!chain_wait(a, s, k, n, limit, t)) return false;
-      load_tile(a, k, k + 1, s.As, t);
-      if (limit > 0) load_tile(a, k + 1, k + 1, s.Bs, t);               // (helping out may have overwritten Bs)
-      load_diag();
-      __syncthreads();
-      product(s.As, s.Bs, acc, tx, ty);
-      __syncthreads();
-      float* out = a.A + (int64_t)(TB * k + ty) * a.ld + TB * (k + 1) + tx;
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          s.As[ty + 16 * p][tx + 16 * q] = acc[p][q];
-          if (TB * (k + 1) + tx + 16 * q < a.w) out[(int64_t)(16 * p) * a.ld + 16 * q] = acc[p][q];
-        }
-      __syncthreads();
-      if (t == 0) { st_release(&a.fl->solved[k * kMaxTiles + k + 1], 1); }
-      product<true>(s.As, s.As, acc, tx, ty);
+    const bool paired = !(k & 1) && k + 1 < nt;          // with column k + 1
+    bool helped = false;
+    const int limit = tasks_before_step(nt, k + 1);
+    if (k < nt - 1 && !chain_wait(a, s, k, nt - 2 - k, limit, t, helped)) return false;
+    if (paired) {
+      if (helped) load_pair_tile(pair_tile(a, k, kPairV1), s.D, t);
+      pair_step(a, s, k, t);
     } else {
-      load_diag();
+      float old[4][4], acc[4][4];
+      const float* Mkk = a.A + (int64_t)(TB * k + ty) * a.ld + TB * k + tx;
+      auto load_diag = [&]() {
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int r = ty + 16 * p, c = tx + 16 * q;
+            old[p][q] = r == c ? 1.f : 0.f;                             // rows beyond the block: identity
+            if (TB * k + r < a.w && TB * k + c < a.w && r <= c) old[p][q] = __ldcg(Mkk + (int64_t)(16 * p) * a.ld + 16 * q);
+            acc[p][q] = 0.f;
+          }
+      };
+      if (k < nt - 1) {
+        // T[k][k + 1] = M[k][k + 1] V^T, and its update of tile (k, k).  (Bs holds V_{k+1}, left there by the last step.)
+        load_tile(a, k, k + 1, s.As, t);
+        if (limit > 0) load_tile(a, k + 1, k + 1, s.Bs, t);             // (helping out may have overwritten Bs)
+        load_diag();
+        __syncthreads();
+        product(s.As, s.Bs, acc, tx, ty);
+        __syncthreads();
+        float* out = a.A + (int64_t)(TB * k + ty) * a.ld + TB * (k + 1) + tx;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            s.As[ty + 16 * p][tx + 16 * q] = acc[p][q];
+            if (TB * (k + 1) + tx + 16 * q < a.w) out[(int64_t)(16 * p) * a.ld + 16 * q] = acc[p][q];
+          }
+        __syncthreads();
+        if (t == 0) { st_release(&a.fl->solved[k * kMaxTiles + k + 1], 1); }
+        product<true>(s.As, s.As, acc, tx, ty);
+      } else {
+        load_diag();
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s.D[ty + 16 * p][tx + 16 * q] = (double)old[p][q] - (double)acc[p][q];
+      __syncthreads();
     }
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) s.D[ty + 16 * p][tx + 16 * q] = (double)old[p][q] - (double)acc[p][q];
-    __syncthreads();
     factor64(s, t, a.k_global + TB * k, a.dev_info);
 #pragma unroll
     for (int p = 0; p < 4; ++p)
@@ -403,6 +544,14 @@ __device__ __forceinline__ bool run_chain(const Args& a, Smem& s, int t) {
       }
     __syncthreads();
     if (t == 0) st_release(&a.fl->factored, nt - k);
+    // the inverse in fp64, for the pair (off the chain: what waits for it has most of a step's time)
+    if (k & 1) {
+      store_pair_tile(pair_tile(a, k, kPairV1), s.D, t);
+    } else if (paired) {
+      store_pair_tile(pair_tile(a, k, kPairV0), s.D, t);
+      __syncthreads();
+      if (t == 0) st_release(&a.fl->paired[k >> 1], 1);
+    }
   }
   return true;
 }
@@ -445,9 +594,10 @@ __global__ void __launch_bounds__(256) panel_place_inverse_kernel(float* __restr
 }
 
 // Factors and inverts the w x w block at A (leading dimension ld) on stream s: its upper triangle holds V = T^-1
-// afterwards, zeros below.  `fl` must be all zero and is left so.  max_ctas: how many CTAs may be spent on it.
-inline gptq_status_t launch(float* A, int64_t ld, int w, int k_global, Flags* fl, int* dev_info, int max_ctas, cudaStream_t s) {
-  Args a{A, ld, w, ceil_div(w, TB), k_global, fl, dev_info};
+// afterwards, zeros below.  `fl` must be all zero and is left so; `pairs`: pair_doubles(w) of scratch.  max_ctas: how many CTAs
+// may be spent on it.
+inline gptq_status_t launch(float* A, int64_t ld, int w, int k_global, Flags* fl, double* pairs, int* dev_info, int max_ctas, cudaStream_t s) {
+  Args a{A, ld, w, ceil_div(w, TB), k_global, fl, pairs, dev_info};
   const int products = tasks_before_step(a.nt, -1);
   // no more CTAs than the widest step has products
   int widest = 1;
