@@ -81,6 +81,7 @@ struct StripeBars {
   uint64_t stage_full[kStripeStages], stage_empty[kStripeStages];     // far panel
   uint64_t acc_full[2], acc_empty[2];         // far accumulators
   uint64_t next_ready[2], all_ready[2];       // the far pushes have reached memory: onto the block after next / all
+  uint64_t settled[2];                        // everything that the near / the far pushes have issued is over
   uint32_t tmem;
 };
 constexpr int kStripeSmem = 1024 + kStripeOffBars + (int)sizeof(StripeBars);
@@ -276,6 +277,20 @@ __device__ __forceinline__ bool stripe_wait(uint64_t* bar, int phase, bool& ok, 
   return ok;
 }
 
+// The last thing an issuing thread does, however it got there: it waits for what it has in flight, so that shared and tensor memory
+// are not given up under a load or an instruction that still uses them -- its MMAs and their commits by one more commit, and the
+// last loads into its ring.  These end by themselves, so the limit is a fixed one, not the adjustable one of the roles' waits.
+__device__ __forceinline__ void stripe_settle(uint64_t* settled, uint64_t* ring_full, int stages, int loaded, int* dev_info, int code) {
+  auto wait = [&](uint64_t* b, uint32_t parity) {
+    const uint64_t t0 = umma::global_timer_ns();
+    while (!umma::mbar_try_wait(b, parity))
+      if (umma::global_timer_ns() - t0 > 1000000000ull) { report_error(dev_info, GPTQ_ERR_TIMEOUT, code); return; }
+  };
+  umma::mma_commit(settled);
+  wait(settled, 0u);
+  for (int m = loaded > stages ? loaded - stages : 0; m < loaded; ++m) wait(&ring_full[m % stages], (uint32_t)(m / stages) & 1u);
+}
+
 // Warp 6: the 16 x 16 diagonal blocks of U as doubles, 1 / U_jj, sK and 1 / sC, one sub-block ahead of the row warps.
 __device__ __forceinline__ void stripe_stage_cols(const StripeArgs& a, StripeCols* cols, StripeBars& bar, int lane) {
   const int n_sub = a.nb2 / kStripeSB;
@@ -310,9 +325,9 @@ __device__ __forceinline__ void stripe_stage_cols(const StripeArgs& a, StripeCol
   }
 }
 
-// Warp 4, one lane: after every 16 columns, their errors onto the rest of the block and onto the next block.
+// Warp 4, one lane: after every 16 columns, their errors onto the rest of the block and onto the next block.  loaded: slices asked for.
 __device__ __forceinline__ void stripe_push_near(const StripeMaps& maps, const StripeArgs& a, uint8_t* etiles, uint8_t* slices,
-                                                 StripeBars& bar, uint32_t tmem) {
+                                                 StripeBars& bar, uint32_t tmem, int& loaded) {
   using namespace umma;
   bool ok = true;
   auto load = [&](int b, int s, int n) -> bool {
@@ -320,6 +335,7 @@ __device__ __forceinline__ void stripe_push_near(const StripeMaps& maps, const S
     const int j0 = s * kStripeSB, boxes = (k.width - j0 - kStripeSB + k.next + 31) / 32;
     if (!stripe_wait(&bar.slice_empty[n & 1], (n >> 1) ^ 1, ok, a.dev_info, 31)) return false;
     uint8_t* dst = slices + (n & 1) * 2 * kStripeSlice;
+    loaded = n + 1;
     mbar_arrive_expect_tx(&bar.slice_full[n & 1], (uint32_t)boxes * 2048);
     for (int q = 0; q < boxes; ++q) {
       tma_load_2d(dst + 1024 * q, &maps.s_hi, a.i2 + k.ib + j0, k.ib + j0 + kStripeSB + 32 * q, &bar.slice_full[n & 1]);
@@ -364,9 +380,9 @@ __device__ __forceinline__ void stripe_push_near(const StripeMaps& maps, const S
   }
 }
 
-// Warp 5, one lane: a block's errors onto the columns after the next block.
+// Warp 5, one lane: a block's errors onto the columns after the next block.  loaded: K atoms asked for.
 __device__ __forceinline__ void stripe_push_far(const StripeMaps& maps, const StripeArgs& a, uint8_t* etiles, uint8_t* stages,
-                                                StripeBars& bar, uint32_t tmem) {
+                                                StripeBars& bar, uint32_t tmem, int& loaded) {
   using namespace umma;
   bool ok = true;
   const int n_atoms = (a.B + 63) >> 6;                    // 64-wide K atoms in a block
@@ -379,6 +395,7 @@ __device__ __forceinline__ void stripe_push_far(const StripeMaps& maps, const St
       const int st = hh % kStripeStages, x = a.i2 + k.ib + 64 * (u % n_atoms), y = col0 + u / n_atoms * kStripeNT;
       if (!stripe_wait(&bar.stage_empty[st], (hh / kStripeStages) ^ 1, ok, a.dev_info, 32)) return false;
       uint8_t* sp = stages + st * kStripeStage;
+      loaded = hh + 1;
       mbar_arrive_expect_tx(&bar.stage_full[st], (uint32_t)kStripeStage);
       tma_load_2d(sp, &maps.p_hi, x, y, &bar.stage_full[st]);
       tma_load_2d(sp + 8192, &maps.p_lo, x, y, &bar.stage_full[st]);
@@ -482,6 +499,7 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
     }
     for (int s = 0; s < kStripeStages; ++s) { mbar_init(&bar.stage_full[s], 1); mbar_init(&bar.stage_empty[s], 1); }
     mbar_init(&bar.errors, 4); mbar_init(&bar.near_done, 1); mbar_init(&bar.rest_done, 1);
+    mbar_init(&bar.settled[0], 1); mbar_init(&bar.settled[1], 1);
     fence_barrier_init();
     fence_proxy_async();
     prefetch_tmap(&maps.p_hi); prefetch_tmap(&maps.p_lo); prefetch_tmap(&maps.s_hi); prefetch_tmap(&maps.s_lo);
@@ -497,9 +515,16 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
     stripe_drain_far(a, bar, tmem, warp & 3, lane);
   } else if (warp >= 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 112;");
-    if (warp == 4) { if (lane == 0) stripe_push_near(maps, a, base, base + kStripeOffSlice, bar, tmem); }
-    else if (warp == 5) { if (lane == 0) stripe_push_far(maps, a, base, base + kStripeOffFar, bar, tmem); }
-    else if (warp == 6) stripe_stage_cols(a, cols, bar, lane);
+    int loaded = 0;
+    if (warp == 4 && lane == 0) {
+      stripe_push_near(maps, a, base, base + kStripeOffSlice, bar, tmem, loaded);
+      stripe_settle(&bar.settled[0], bar.slice_full, 2, loaded, a.dev_info, 46);
+    } else if (warp == 5 && lane == 0) {
+      stripe_push_far(maps, a, base, base + kStripeOffFar, bar, tmem, loaded);
+      stripe_settle(&bar.settled[1], bar.stage_full, kStripeStages, loaded, a.dev_info, 47);
+    } else if (warp == 6) {
+      stripe_stage_cols(a, cols, bar, lane);
+    }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 248;");
     // ---------------------------------------------------------------- the rows, one thread each

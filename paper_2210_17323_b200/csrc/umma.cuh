@@ -50,11 +50,15 @@ constexpr uint64_t kWaitLimitNs = 4000000000ull;  // 4 s: far beyond any legitim
 static __device__ unsigned long long g_wait_limit_ns = kWaitLimitNs;
 static __device__ int g_skip_loads_of_item = -1;
 
+// The contraction kernels' roles leave at once after a wait that ran out: their own copies in flight are then as old as the wait,
+// and over.  So no test sets their limit below a millisecond.
+__device__ __forceinline__ uint64_t contraction_wait_limit() { return g_wait_limit_ns < 1000000ull ? 1000000ull : g_wait_limit_ns; }
+
 // Waits for the phase with the given parity; false if the limit ran out.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_timer_ns();
-  const uint64_t limit = g_wait_limit_ns;
+  const uint64_t limit = contraction_wait_limit();
   uint32_t spins = 0;
   while (!mbar_try_wait(bar, parity)) {
     if ((++spins & 0x3FF) == 0 && global_timer_ns() - t0 > limit) return false;

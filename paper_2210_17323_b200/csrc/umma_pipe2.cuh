@@ -73,7 +73,7 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
   if (mbar_try_wait_cluster(bar, parity)) return true;
   const uint64_t t0 = umma::global_timer_ns();
-  const uint64_t limit = umma::g_wait_limit_ns;
+  const uint64_t limit = umma::contraction_wait_limit();
   uint32_t spins = 0;
   while (!mbar_try_wait_cluster(bar, parity)) {
     if ((++spins & 0x3FF) == 0 && umma::global_timer_ns() - t0 > limit) return false;

@@ -720,6 +720,34 @@ def test_bounded_waits_report_timeout_and_the_gpu_stays_usable(B, D):
     assert rel_fro(H.cpu().numpy(), Href) <= TOL_H_FRO
 
 
+@pytest.mark.parametrize("R,C,bits,group,block", [(200, 1024, 4, 0, 128), (130, 768, 3, 8, 64), (128, 960, 3, 192, 96)])
+def test_waits_of_the_row_stripes_report_timeout_and_the_next_call_is_right(B, R, C, bits, group, block):
+    """With a limit of a nanosecond every role of the row-stripe kernel leaves at its first wait that is not over already: the call reports
+    it and ends by itself, and the next one, with the limit back and in the same workspace, gives what it gave before."""
+    L = _layer(R, C, 2 * C, cfg=11)
+    W = torch.from_numpy(L.w()).cuda()
+    H = torch.from_numpy(O.hessian_accumulate(np.zeros((C, C)), L.x_bits()).astype(np.float32)).cuda()
+    U, _ = B.gptq_prepare_hinv(H, 0.01)
+    ws = torch.empty(B.gptq_quantize_workspace_bytes(R, C, bits, group, block), dtype=torch.uint8, device="cuda")
+    ref = B.gptq_quantize_layer(W, U, bits, group, False, block, ws=ws)
+    torch.cuda.synchronize()
+    assert ref["dev_info"].tolist() == [0, 0]
+    try:
+        B.gptq_debug_wait_test(1, -1)
+        out = B.gptq_quantize_layer(W, U, bits, group, False, block, ws=ws)
+        torch.cuda.synchronize()
+        status, code = out["dev_info"].tolist()
+        assert status == B.ERR_TIMEOUT and 31 <= code <= 45, (status, code)
+    finally:
+        B.gptq_debug_wait_test(0, -1)
+    out = B.gptq_quantize_layer(W, U, bits, group, False, block, ws=ws)
+    torch.cuda.synchronize()
+    assert out["dev_info"].tolist() == [0, 0]
+    for key in ("qweight", "zeros"):
+        assert torch.equal(out[key], ref[key])
+    assert rel_fro(out["scales"].cpu().numpy(), ref["scales"].cpu().numpy()) <= 1e-6
+
+
 def test_solve_layer_from_host_buffers_several_grids(B):
     """One host-buffer call for several grids of a layer (activations cross once, one Hessian and factor): every grid's
     result matches the oracle, and equals the single-grid call's for the grid they share."""
