@@ -123,6 +123,8 @@ gptq_status_t gptq_hessian_symmetrize(float* H, int C, void* stream);
  *            the factor or of its inverse left the range of the scaled fp16 operand pairs the
  *            tensor-core contractions use for C > 1024 (a Hessian so ill-conditioned that entries of
  *            the inverse factor exceed ~100 times their row's diagonal entry); [1] = a row index.
+ *            GPTQ_ERR_TIMEOUT, at any C: a bounded wait inside one of the kernels ran out and U is not
+ *            the factor; [1] = which wait (61, 62: the panel launch; others: the contractions).
  * Computed as the inverse of the upper factor of H~ = U~ U~^T, which equals
  * Cholesky(H~^-1)^T by uniqueness of the Cholesky factor.
  * Streams: for C > 1024 part of the work is enqueued on an internal stream (created once

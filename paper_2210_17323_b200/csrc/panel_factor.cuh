@@ -84,7 +84,7 @@ __device__ __forceinline__ bool wait_ge(const int* p, int v, const Args& a) {
     if ((spins & 0x3F) == 0) {
       if (ld_acquire(&a.fl->abort)) return false;
       if (umma::global_timer_ns() - t0 > limit) {
-        report_error(a.dev_info, GPTQ_ERR_TIMEOUT, 41);
+        report_error(a.dev_info, GPTQ_ERR_TIMEOUT, 61);
         st_release(&a.fl->abort, 1);
         return false;
       }
@@ -401,7 +401,7 @@ __device__ __forceinline__ bool chain_wait(const Args& a, Smem& s, int k, int n,
       if (t0 == 0) t0 = now;
       if (ld_acquire(&a.fl->abort)) m = 3;
       else if (now - t0 > umma::g_wait_limit_ns) {
-        report_error(a.dev_info, GPTQ_ERR_TIMEOUT, 42);
+        report_error(a.dev_info, GPTQ_ERR_TIMEOUT, 62);
         st_release(&a.fl->abort, 1);
         m = 3;
       } else if (now - t0 > 20000) {

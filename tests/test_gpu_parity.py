@@ -748,6 +748,29 @@ def test_waits_of_the_row_stripes_report_timeout_and_the_next_call_is_right(B, R
     assert rel_fro(out["scales"].cpu().numpy(), ref["scales"].cpu().numpy()) <= 1e-6
 
 
+@pytest.mark.parametrize("C", [96, 320, 1024])
+def test_waits_of_the_panel_launch_report_timeout_and_the_next_call_is_right(B, C):
+    """With a limit of a nanosecond the first wait of any CTA that is not over already abandons the panel launch: the call reports it and
+    ends by itself; the next one, with the limit back and in the same workspace (its progress words were left in the middle of
+    things), gives what it gave before, bit for bit."""
+    H = torch.from_numpy(O.hessian_accumulate(np.zeros((C, C)), _layer(8, C, 2 * C, cfg=12).x_bits()).astype(np.float32)).cuda()
+    ws = torch.empty(B.gptq_prepare_hinv_workspace_bytes(C), dtype=torch.uint8, device="cuda")
+    ref, info = B.gptq_prepare_hinv(H, 0.01, ws=ws)
+    torch.cuda.synchronize()
+    assert info.tolist() == [0, 0]
+    try:
+        B.gptq_debug_wait_test(1, -1)
+        _, info = B.gptq_prepare_hinv(H, 0.01, ws=ws)
+        torch.cuda.synchronize()
+        status, code = info.tolist()
+        assert status == B.ERR_TIMEOUT and code in (61, 62), (status, code)
+    finally:
+        B.gptq_debug_wait_test(0, -1)
+    U, info = B.gptq_prepare_hinv(H, 0.01, ws=ws)
+    torch.cuda.synchronize()
+    assert info.tolist() == [0, 0] and torch.equal(U, ref)
+
+
 def test_solve_layer_from_host_buffers_several_grids(B):
     """One host-buffer call for several grids of a layer (activations cross once, one Hessian and factor): every grid's
     result matches the oracle, and equals the single-grid call's for the grid they share."""
