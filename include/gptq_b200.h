@@ -77,8 +77,9 @@ uint64_t gptq_launch_count(void);
  * kernel records GPTQ_ERR_TIMEOUT in dev_info, every role leaves through its own bounded wait, tensor memory is freed and
  * the kernel returns -- it never hangs or traps.  This call lets a test see that path: it sets the limit of the waits
  * (nanoseconds; 0 restores the default of 4 s; the contraction kernels take no less than a millisecond) and the index of
- * one work item whose operand loads the producer leaves out (-1: none), for kernels of the current device launched
- * afterwards.  Synchronises the device.  Restore with (0, -1). */
+ * one work item whose operand loads the producer leaves out (-1: none; -2: none, but in stage 2's panel launches every CTA
+ * except the one that runs the dependency chain leaves at once, so that it does all the work), for kernels of the current
+ * device launched afterwards.  Synchronises the device.  Restore with (0, -1). */
 gptq_status_t gptq_debug_wait_test(uint64_t wait_limit_ns, int skip_loads_of_item);
 
 /* ------------------------------------------------------------------ stage 1

@@ -99,7 +99,8 @@ def gptq_launch_count() -> int:
 
 
 def gptq_debug_wait_test(wait_limit_ns=0, skip_loads_of_item=-1):
-    """Test hook: limit of the kernels' bounded waits and one work item whose loads are left out; (0, -1) restores."""
+    """Test hook: limit of the kernels' bounded waits and one work item whose loads are left out (-2: the panel launches' chain
+    CTA works alone); (0, -1) restores."""
     st = _lib.gptq_debug_wait_test(int(wait_limit_ns), int(skip_loads_of_item))
     if st != OK:
         raise GptqError(st, "gptq_debug_wait_test")

@@ -564,6 +564,7 @@ __global__ void __launch_bounds__(kThreads, 2) panel_factor_kernel(const Args a)
   __syncthreads();
   const bool chain = s.msg[0] == 0;
   __syncthreads();
+  if (!chain && umma::g_skip_loads_of_item == umma::kPanelChainAlone) return;       // (test knob)
   if (chain && !run_chain(a, s, t)) return;
   for (;;) {
     if (t == 0) s.msg[0] = atomicAdd(&a.fl->ticket, 1);

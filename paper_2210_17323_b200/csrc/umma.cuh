@@ -49,6 +49,7 @@ constexpr uint64_t kWaitLimitNs = 4000000000ull;  // 4 s: far beyond any legitim
 // index of one work item whose operand loads the producer leaves out, so that the waits downstream of it run out.
 static __device__ unsigned long long g_wait_limit_ns = kWaitLimitNs;
 static __device__ int g_skip_loads_of_item = -1;
+constexpr int kPanelChainAlone = -2;              // as that index: in panel launches every CTA but the first leaves at once
 
 // The contraction kernels' roles leave at once after a wait that ran out: their own copies in flight are then as old as the wait,
 // and over.  So no test sets their limit below a millisecond.

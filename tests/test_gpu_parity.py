@@ -771,6 +771,25 @@ def test_waits_of_the_panel_launch_report_timeout_and_the_next_call_is_right(B, 
     assert info.tolist() == [0, 0] and torch.equal(U, ref)
 
 
+@pytest.mark.parametrize("C", [128, 224, 640, 1024, 1120])
+def test_panel_launch_needs_no_second_cta(B, C):
+    """The CTA that runs the chain takes the list's products itself where nobody else does, so nothing rests on CTAs being resident
+    together.  The same products in the same order: bit for bit the result of the whole grid (beyond 1024 columns up to the order of
+    the contractions' sums in memory)."""
+    H = torch.from_numpy(O.hessian_accumulate(np.zeros((C, C)), _layer(8, C, 2 * C, cfg=13).x_bits()).astype(np.float32)).cuda()
+    ref, info = B.gptq_prepare_hinv(H, 0.01)
+    torch.cuda.synchronize()
+    assert info.tolist() == [0, 0]
+    try:
+        B.gptq_debug_wait_test(0, -2)
+        U, info = B.gptq_prepare_hinv(H, 0.01)
+        torch.cuda.synchronize()
+    finally:
+        B.gptq_debug_wait_test(0, -1)
+    assert info.tolist() == [0, 0]
+    assert torch.equal(U, ref) if C <= 1024 else rel_fro(U.cpu().numpy(), ref.cpu().numpy()) <= 1e-6
+
+
 def test_solve_layer_from_host_buffers_several_grids(B):
     """One host-buffer call for several grids of a layer (activations cross once, one Hessian and factor): every grid's
     result matches the oracle, and equals the single-grid call's for the grid they share."""
