@@ -121,8 +121,8 @@ def test_prepare_hinv_matches_oracle(B, C):
 
 @pytest.mark.parametrize("R,group,bits", [(130, 0, 4), (128, 32, 3), (1, 8, 2), (257, 128, 8)])
 def test_quantize_weights_on_ties(B, R, group, bits):
-    """Weights halfway between two codes (and, once per row, far outside everything else): the column loop decides such columns with the
-    division itself.  With a diagonal H nothing moves a weight, so the codes are the oracle's nearest codes exactly."""
+    """Weights halfway between two codes: the column loop decides such columns with the division itself.  With a diagonal H nothing moves a
+    weight, so the codes are the oracle's nearest codes exactly."""
     C = 256
     rng = np.random.default_rng(bits)
     maxq = 2 ** bits - 1
@@ -134,6 +134,39 @@ def test_quantize_weights_on_ties(B, R, group, bits):
     ref = O.quantize_layer(W, np.eye(C), bits, group, False, 128)
     assert np.array_equal(O.unpack_codes(out["qweight"].view(np.uint32), bits, C), ref["codes"])
     assert np.array_equal(out["scales"], ref["scales"].astype(np.float32)) and np.array_equal(out["zeros"], ref["zeros"])
+
+
+@pytest.mark.parametrize("R,group,bits", [(130, 0, 4), (33, 32, 3), (128, 16, 2), (65, 64, 8)])
+def test_quantize_weights_on_the_ties_of_a_symmetric_grid(B, R, group, bits):
+    """The same for a symmetric grid, whose lower end is a tie too: every weight a multiple of half a step, every group's largest weight
+    the upper end of the grid."""
+    C, maxq = 256, 2 ** bits - 1
+    W = (np.random.default_rng(bits).integers(-maxq, maxq + 1, (R, C)) * 2.0 ** -7).astype(np.float16)
+    W[:, ::group if group > 0 else C] = maxq * 2.0 ** -7                                        # scale 2^-6
+    out = _run_quant(B, W, np.eye(C, dtype=np.float32), bits, group, True, 128)
+    ref = O.quantize_layer(W, np.eye(C), bits, group, True, 128)
+    assert np.array_equal(O.unpack_codes(out["qweight"].view(np.uint32), bits, C), ref["codes"])
+    assert np.array_equal(out["scales"], ref["scales"].astype(np.float32)) and np.array_equal(out["zeros"], ref["zeros"])
+
+
+def test_quantize_weights_far_outside_their_grid(B):
+    """Feedback that carries weights more than 2048 steps off their 8-bit grid, to both sides, where the column loop's fixed-point quotient
+    has no room and the division decides: inside the sixteen columns of the error that does it, in the next sixteen, in the next
+    block and two blocks on.  (Fewer bits would take the errors out of the fp16 pairs' range first, which the call reports.)"""
+    R, C, a = 130, 512, 0.5
+    rng = np.random.default_rng(3)
+    W = rng.uniform(-a, a, (R, C)).astype(np.float16)
+    W[:, 1], W[:, 2] = -a, a                                       # scale 2 a / 255
+    step = 2 * a / 255
+    W[:, 0] = ((rng.integers(-20, 20, R) + np.where(np.arange(R) % 2, 0.3, -0.3)) * step).astype(np.float16)
+    U = np.eye(C, dtype=np.float32)
+    far = [5, 20, 150, 300, 511]
+    U[0, far] = np.float32(2600.0 / 0.3) * np.array([1, -1, 1, -1, 1], dtype=np.float32)      # about 2600 steps
+    out = _run_quant(B, W, U, 8, 0, False, 128)
+    ref = O.quantize_layer(W, U.astype(np.float64), 8, 0, False, 128)
+    assert (np.abs(ref["E"][:, far]) > 2048 * step).all() and set(np.unique(ref["codes"][:, far])) == {0, 255}
+    assert np.array_equal(O.unpack_codes(out["qweight"].view(np.uint32), 8, C), ref["codes"])
+    assert abs(out["loss"] - ref["loss"]) <= 1e-5 * ref["loss"]
 
 
 @pytest.mark.parametrize("R,C,bits,group,block", [
