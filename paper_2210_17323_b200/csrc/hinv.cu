@@ -384,7 +384,7 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
 
   // Phase 1: backwards blocked Cholesky H~ = U~ U~^T in U's upper triangle, outer panels of kNB2 columns
   // from the last to the first, left-looking: a panel receives the contributions of all later columns in
-  // one contraction over the tf32 hi / lo copies F of the finished factor.  Per panel J (rows j0..rows_p
+  // one contraction over the fp16 hi / lo copies F of the finished factor.  Per panel J (rows j0..rows_p
   // are its diagonal block D, "row block J-1" are the kNB2 rows above D):
   //   chain stream                                         wide stream
   //   C1  D -= F[J rows, later] F[J rows, later]^T         B1  A[0:j0, J] -= F[0:j0, later] F[J rows, later]^T

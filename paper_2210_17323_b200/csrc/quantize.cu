@@ -636,7 +636,7 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
   if (factor && C > GPTQ_FACTOR_BLOCK && (!stripe || B2 != GPTQ_FACTOR_BLOCK)) return GPTQ_ERR_UNSUPPORTED;
   for (int i2 = 0; i2 < C; i2 += B2) {
     const int nb2 = (C - i2 < B2) ? C - i2 : B2;
-    {  // transposed tf32 hi/lo pair of U[0 : i2 + nb2, i2 : i2 + nb2] for the contractions of this outer block
+    {  // transposed fp16 hi / lo pair of U[0 : i2 + nb2, i2 : i2 + nb2] for the contractions of this outer block
       dim3 grid(nb2 / 32, ceil_div(i2 + nb2, 128)), blk(32, 8);
       split_panel_t_kernel<<<grid, blk, 0, s>>>(U, C, i2, i2 + nb2, sK, sC, factor ? sC2 : nullptr, Phi, Plo, (int64_t)C);
       GPTQ_LAUNCH_CHECK();
@@ -741,10 +741,3 @@ extern "C" int gptq_set_stage3_variant(int variant) {
   if (variant != 0 && variant != 1) return gptq::g_stage3_variant.load();
   return gptq::g_stage3_variant.exchange(variant);
 }
-
-#ifdef GPTQ_EXP_TIMING
-extern "C" int gptq_dbg_stripe_timing(unsigned long long* out32, int reset) {
-  if (reset) { unsigned long long z[32] = {}; return (int)cudaMemcpyToSymbol(gptq::g_stripe_dbg, z, sizeof(z)); }
-  return (int)cudaMemcpyFromSymbol(out32, gptq::g_stripe_dbg, 32 * sizeof(unsigned long long));
-}
-#endif

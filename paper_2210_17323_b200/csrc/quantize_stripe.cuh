@@ -29,8 +29,9 @@
 //
 // Threads: warps 0-3 own the rows (thread t <-> row t <-> TMEM lane t); warp 4 issues the near pushes, warp 5 the far ones,
 // warp 6 stages U's diagonal blocks, warp 7 has nothing to do, warps 8-11 drain the far pushes.  A row thread needs 200
-// registers and more (32 doubles of weights); spilled, the loads that run ahead are waited for.  So the three warpgroups
-// share out the registers anew: 248 + 112 + 136 of the 3 x 168 the kernel is launched with.
+// registers and more (32 doubles of weights); at 168 the loads that run ahead are spilled, and so waited for.  So the three
+// warpgroups share out the registers anew: 248 + 112 + 136 of the 3 x 168 the kernel is launched with.  (The instance without
+// small groups still spills 20 bytes somewhere, the other one none.)
 #pragma once
 
 constexpr int kStripeRows = 128;
@@ -139,19 +140,9 @@ __device__ __noinline__ double column_by_division(double w, double scale, double
   return (w - scale * (q - zero)) * rdiag;
 }
 
-#ifdef GPTQ_EXP_TIMING
-__device__ unsigned long long g_stripe_dbg[32];
-#define TICK(var) long long var = clock64()
-#define TOCK(slot, var) do { const long long z_ = clock64(); if (blockIdx.x == 0 && (threadIdx.x & 31) == 0 && (warp == 0 || warp == 8)) atomicAdd(&g_stripe_dbg[slot], (unsigned long long)(z_ - (var))); (var) = z_; } while (0)
-#else
-#define TICK(var)
-#define TOCK(slot, var)
-#endif
-
-
 // ---- pieces of the row threads' loop ------------------------------------------------------------------
 // Sixteen columns of the working weights as memory holds them (rows beyond the matrix: zero, so that nothing of them is ever
-// pushed).  Bulk reductions of this launch changed them, so L1 is bypassed.
+// pushed).  Reductions of this launch changed them, so L1 is bypassed.
 __device__ __forceinline__ void stripe_fetch(const double* wcol, bool live, double (&x)[kStripeSB]) {
 #pragma unroll
   for (int m = 0; m < kStripeSB; ++m) x[m] = live ? __ldcg(wcol + (int64_t)m * kStripeRows) : 0.0;
@@ -544,7 +535,6 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
     double ahead[kStripeSB];                              // the next sixteen columns, on their way
     stripe_fetch(wg, live, ahead);
     int n = 0;                                            // sub-blocks so far
-    TICK(tk);
 #pragma unroll 1
     for (int b = 0; b * a.B < a.nb2; ++b) {
       const StripeBlock k = stripe_block(a, b);
@@ -560,7 +550,6 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
         stripe_wait(&bar.cols_full[n & 1], n >> 1, ok, a.dev_info, 36);
         if (n > 0) stripe_wait(&bar.near_done, n - 1, ok, a.dev_info, 37);
         fence_after_thread_sync();
-        TOCK(0, tk);
         if (g >= 32 && ((i + j0) % g) == 0) {              // a group starts (wider than the block: only at j0 = 0)
           if (g > a.B) {
             const int q = min(b - 1, (a.nb2 + a.B - 1) / a.B - 3);        // the last block before this one with far pushes
@@ -573,7 +562,6 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
           grid.set(sz, a.grid.maxq);
           if (live) { a.scales[(int64_t)row * G + (i + j0) / g] = sz.x; a.zeros[(int64_t)row * G + (i + j0) / g] = sz.y; }
         }
-        TOCK(1, tk);
         double w[kStripeSB];
 #pragma unroll
         for (int m = 0; m < kStripeSB; ++m) w[m] = ahead[m];
@@ -585,7 +573,6 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
           if (j0 + kStripeSB == k.width && b >= 1 && col < a.nb2) stripe_wait(&bar.next_ready[(b - 1) & 1], (b - 1) >> 1, ok, a.dev_info, 44);
           if (col < a.nb2) stripe_fetch(wg + (int64_t)col * kStripeRows, live, ahead);
         }
-        TOCK(2, tk);
         StripeGroups sg{g, small_group_starts, a.grid, a.scales + (int64_t)row * G + (i + j0) / (g > 0 ? g : 1),
                         a.zeros + (int64_t)row * G + (i + j0) / (g > 0 ? g : 1), live};
         // The sixteen columns.  What bounds them is the chain from one column's weight to the next column's, so it is kept to
@@ -626,7 +613,6 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
           for (int m = 0; m < kStripeSB / 4; ++m) cw[m] = r.cw[m];
           l0 = r.loss;
         }
-        TOCK(3, tk);
         // scaled errors as an fp16 hi / lo pair: into the swizzled K-major tile (row t, 16-byte chunk (k / 8) ^ (t & 7) of
         // the 128-byte row of K atom k / 64) and, in the inverse form, to global memory for the left-looking contractions of
         // later outer blocks; codes as bytes
@@ -666,7 +652,6 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
           }
           *reinterpret_cast<uint4*>(a.codes + o) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
         }
-        TOCK(4, tk);
       }
     }
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, o);
