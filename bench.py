@@ -493,8 +493,8 @@ def run_gpu(args, wl):
              peak=f16_peak, unit="TFLOP/s", frac=3 * fac_ach / f16_peak, useful_frac=fac_ach / f16_peak,
              flops=("useful C^3 / 3 for the layers in the factor form (the backwards factorisation alone), 2 C^3 / 3 for the others"
                     if factor else "useful 2 C^3 / 3") +
-                   "; executed = 3 x (hi*hi + hi*lo + lo*hi); the serial 128 x 128 diagonal-block chain and the "
-                   "CUDA-core work inside an outer panel are inside this time"),
+                   "; executed = 3 x (hi*hi + hi*lo + lo*hi); the panel launches (serial chain of 64 x 64 fp64 tiles, "
+                   "CUDA-core tile products) are inside this time"),
         dict(stage="quantize_layer", bound="tensor", dtype="fp16 pairs, 3 products per term", achieved=upd_ach, executed=3 * upd_ach,
              peak=f16_peak, unit="TFLOP/s", frac=3 * upd_ach / f16_peak, useful_frac=upd_ach / f16_peak,
              flops="useful R (C^2 - C B) per grid (lazy updates)" + (" + R C 1024 (the blocks' own U, factor form)" if factor else "") +

@@ -19,7 +19,8 @@
 // chain, if what it waits for has not been taken by anybody, takes it itself (chain_wait).  Every wait is bounded.
 // As separate launches (one 128-wide diagonal kernel of 97 us, two small GEMMs, two more on a side stream for the
 // inverse, per 128 columns) a 1024-wide call took 1.29 ms; this form 0.254 ms (768 columns: 0.94 -> 0.195 ms), of which the
-// fp64 products of the pairs are 0.006 ms and rsqrt() 0.009.  A chain step is about 15 us.
+// fp64 products of the pairs are 0.006 ms and rsqrt() 0.009.  A chain step is about 15 us; on the chain's SM no pipe is more than
+// half busy (shared memory 46 %, DMMA 16 %).
 #pragma once
 
 namespace gptq {

@@ -69,9 +69,11 @@ __global__ void rtn_pack_kernel(const __half* __restrict__ W, int R, int C, int 
 }
 
 // ---- one pass for groups that are multiples of 32 columns (and per-row grids) -----------------------------------
-// The kernels are bound by issue slots, so what counts is instructions per weight: one for the minimum and maximum (half2),
-// eight for the code.  (12288 x 12288, 4-bit per row: 178 us with single-precision minima and eleven instructions and a
-// branch per code, and one load in flight in the second pass; 112 now, where the bytes alone take 57.)
+// Groups are bound by issue slots (78 % of them filled, 20 instructions a weight with what carries minima and grids between
+// lanes), per-row grids by the latency of their loads and by W's second read, half of which misses L2 (11 instructions a
+// weight, 50 % of the slots).  So: one instruction a weight for the minimum and maximum (half2), few for the code, four loads
+// in flight.  (12288 x 12288, 4-bit per row: 178 us with single-precision minima, a branch per code and one load in flight
+// in the second pass; 113 now, where the bytes alone take 57.)
 __device__ __forceinline__ void rtn_grid_of(float mn, float mx, RtnGrid grid, float& scale, float& zero) {
   double xmin = fmin((double)mn, 0.0), xmax = fmax((double)mx, 0.0);
   if (xmin == 0.0 && xmax == 0.0) { xmin = -1.0; xmax = 1.0; }
