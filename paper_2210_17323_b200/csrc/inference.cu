@@ -92,6 +92,79 @@ dequantize_kernel(const uint32_t* __restrict__ qweight, const float* __restrict_
   }
 }
 
+// ---- whole-matrix dequantization, 16 columns per thread -----------------------------------------------------------
+// Writes dominate (8 bytes of fp16 for every byte of 2-bit codes), and what the memory takes depends on the width of a store:
+// 32 bytes per lane, one instruction, against two or more of 16 (a 2-bit mix of 463 MB alone, without arithmetic: 6.4 against
+// 4.6 TB/s).  Needs a 32-byte aligned output and groups that are multiples of 16 columns; the kernel above does the rest.
+// A thread takes 16 columns of kRows neighbouring rows, whose loads are all in flight before the first is used: four rows where a
+// row's codes are one or two words (14336 x 14336, 2-bit g128, 1 / 2 / 4 rows: 97 / 82 / 76 us, 94 with 16-byte stores; 3-bit 98 / 84 /
+// 80, 117), two for 4 and 8 bits (12288 x 12288, 4-bit: 70 / 60 / 61, 70; 8192 x 8192, 8-bit: 35.1 / 33.3 / 34.1, 39.0).
+template <int F> constexpr int kDqRowsOf = F <= 3 ? 4 : 2;
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+               "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+template <int F>
+__global__ void __launch_bounds__(256)
+dequantize16_kernel(const uint32_t* __restrict__ qweight, const float* __restrict__ scales, const float* __restrict__ zeros,
+                    int R, int C, int g, int G, __half* __restrict__ out) {
+  constexpr int kDqRows = kDqRowsOf<F>;
+  constexpr int kWords = (F + 1) / 2;                         // words that hold the sixteen codes (3-bit: 48 bits from bit 0 or 16 on)
+  const uint32_t chunks = (uint32_t)C / 16, idx = blockIdx.x * 256u + threadIdx.x;
+  const int r0 = (int)(idx / chunks) * kDqRows, ch = (int)(idx % chunks), c0 = 16 * ch;
+  if (r0 >= R) return;
+  const int gi = c0 / g, n = min(kDqRows, R - r0);
+  const int64_t wpr = (int64_t)(C / 32) * F;                  // words per row
+  const uint32_t* q = qweight + r0 * wpr + (ch * F) / 2;
+  uint32_t w[kDqRows][kWords];
+  float s[kDqRows], z[kDqRows];
+#pragma unroll
+  for (int u = 0; u < kDqRows; ++u) {
+    if (u < n) {
+      const uint32_t* p = q + u * wpr;
+      if constexpr (F == 4) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(p)); w[u][0] = v.x; w[u][1] = v.y;
+      } else if constexpr (F == 8) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p)); w[u][0] = v.x; w[u][1] = v.y; w[u][2] = v.z; w[u][3] = v.w;
+      } else {
+#pragma unroll
+        for (int k = 0; k < kWords; ++k) w[u][k] = __ldg(p + k);
+      }
+      s[u] = __ldg(scales + (int64_t)(r0 + u) * G + gi); z[u] = __ldg(zeros + (int64_t)(r0 + u) * G + gi);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kDqRows; ++u) {
+    if (u >= n) break;
+    if constexpr (F == 3) {                                   // the 48 bits to the front
+      if (ch & 1) { w[u][0] = __funnelshift_r(w[u][0], w[u][1], 16); w[u][1] >>= 16; }
+    }
+    uint32_t h[8];
+    // code -> float without an integer conversion: the bit pattern (code | 0x4B000000) is 2^23 + code exactly.  With an integer
+    // zero-point 2^23 + zero is exact too, and their difference is code - zero as it stands.
+    auto bits_of = [&](int i) -> float {
+      const int b = i * F, k = b >> 5, o = b & 31;
+      uint32_t v = w[u][k] >> o;
+      if (o + F > 32) v = __funnelshift_r(w[u][k], w[u][k + 1 < kWords ? k + 1 : k], o);
+      return __uint_as_float((v & ((1u << F) - 1u)) | 0x4B000000u);
+    };
+    auto pair = [&](float a, float b) {
+      const __half2 v = __halves2half2(__float2half_rn(__fmul_rn(s[u], a)), __float2half_rn(__fmul_rn(s[u], b)));
+      return *reinterpret_cast<const uint32_t*>(&v);
+    };
+    if (z[u] == rintf(z[u]) && fabsf(z[u]) <= 4194304.f) {
+      const float base = 8388608.f + z[u];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) h[i] = pair(__fsub_rn(bits_of(2 * i), base), __fsub_rn(bits_of(2 * i + 1), base));
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        h[i] = pair(__fsub_rn(__fsub_rn(bits_of(2 * i), 8388608.f), z[u]), __fsub_rn(__fsub_rn(bits_of(2 * i + 1), 8388608.f), z[u]));
+    }
+    st_global_32(out + (int64_t)(r0 + u) * C + c0, h);
+  }
+}
+
 // ---- y = dequant(Q) x for one fp16 vector x: one warp per row -------------------------------------
 // Lanes take 32-column chunks round-robin.  Per chunk: sq = sum_i q_i x_i, combined with the group's
 // scale and zero as  s * (sq - z * sum_i x_i);  the per-chunk sums of x are computed once per CTA.
@@ -653,6 +726,12 @@ inline bool group_ok(int C, int g) { return g > 0 && C % g == 0 && (g % 32 == 0 
 template <int F>
 gptq_status_t launch_dequantize(const uint32_t* qweight, const float* scales, const float* zeros, int R, int C, int g,
                                 int G, __half* out, cudaStream_t s) {
+  const int64_t threads = (int64_t)((R + gptq::kDqRowsOf<F> - 1) / gptq::kDqRowsOf<F>) * (C / 16);
+  if (g % 16 == 0 && gptq::aligned_to(out, 32) && gptq::aligned_to(qweight, F == 8 ? 16 : F == 4 ? 8 : 4) && threads < 0x7FFFFF00) {
+    gptq::dequantize16_kernel<F><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(qweight, scales, zeros, R, C, g, G, out);
+    GPTQ_LAUNCH_CHECK();
+    return GPTQ_OK;
+  }
   const int gx = (C / 8 + 255) / 256;
   int gy = gptq::device_sm_count() * 32 / gx;                  // about 32 CTAs per SM in total
   if (gy < 1) gy = 1;

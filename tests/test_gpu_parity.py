@@ -1079,3 +1079,26 @@ def test_symmetrize_at_tile_edges(B, C):
     ref = torch.triu(H) + torch.triu(H, 1).T
     B.gptq_hessian_symmetrize(H)
     assert torch.equal(H, ref)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 8, O.BITS_TERNARY])
+@pytest.mark.parametrize("R,C,group", [(1, 32, 0), (3, 32, 16), (5, 96, 48), (257, 1056, 96), (130, 4128, 0), (7, 64, 8)])
+@pytest.mark.parametrize("off", [0, 8])
+def test_dequantize_at_the_edges_of_a_thread(B, bits, R, C, group, off):
+    """Sixteen columns of two or four rows per thread (groups that are multiples of 16, 32-byte aligned output), eight columns otherwise:
+    row counts around multiples of both, one group per thread and many, an output 16 bytes off that boundary, and zero-points that are
+    not integers or beyond 2^22.  Bit for bit what one fp32 subtraction, one fp32 product and one rounding to fp16 give."""
+    rng = np.random.default_rng(R * C + bits)
+    f = 2 if bits == O.BITS_TERNARY else bits
+    G = C // group if group else 1
+    codes = rng.integers(0, 2 ** f, (R, C)).astype(np.uint8)
+    scales = rng.uniform(1e-3, 1e-2, (R, G)).astype(np.float32)
+    zeros = rng.integers(0, 2 ** f, (R, G)).astype(np.float32)
+    zeros[rng.random((R, G)) < 0.2] += 0.375
+    zeros[rng.random((R, G)) < 0.1] = 2.0 ** 23 + 2
+    out = torch.zeros(R * C + 16, dtype=torch.float16, device="cuda")[off:off + R * C].view(R, C)
+    B.gptq_dequantize(torch.from_numpy(O.pack_codes(codes, bits).view(np.int32)).cuda(), torch.from_numpy(scales).cuda(),
+                      torch.from_numpy(zeros).cuda(), C, bits, group, out=out)
+    s, z = np.repeat(scales, C // G, 1), np.repeat(zeros, C // G, 1)
+    want = (s * (codes.astype(np.float32) - z)).astype(np.float16)
+    assert np.array_equal(out.cpu().numpy().view(np.uint16), want.view(np.uint16))
