@@ -60,7 +60,7 @@ struct StripeArgs {
                                               // plain residuals there from the codes
 };
 
-// What the sixteen columns of a sub-block need of U: its diagonal block, 1 / U_jj, sK and 1 / sC.
+// What the sixteen columns of a sub-block need of U: its diagonal block with rows divided by U_jj, 1 / U_jj, sK and 1 / sC.
 struct StripeCols { double U[kStripeSB][kStripeSB]; double rdiag[kStripeSB]; float sks[kStripeSB]; float sci[kStripeSB]; };
 
 // shared memory (from a 1024-byte aligned base):
@@ -125,19 +125,20 @@ __device__ __noinline__ float2 find_params_outofline(double mn, double mx, GridS
 // A row's current grid, with what the column loop derives from it once per grid.
 struct RowGrid {
   double scale, rscale, zero;
-  uint32_t lo, hi;                      // smallest and largest code, counted as the column loop counts them: 2048 - zero-point + code
-  __device__ __forceinline__ void set(float2 sz, int maxq) {
+  double kz;                            // 2^52 + zero-point: what a code's bits with that exponent stand above code - zero-point
+  int bias;                             // what turns the column loop's count, 2048 + code - zero-point, into the code
+  __device__ __forceinline__ void set(float2 sz) {
     scale = (double)sz.x; zero = (double)sz.y; rscale = 1.0 / scale;
-    lo = 2048u - (uint32_t)(int)sz.y; hi = lo + (uint32_t)maxq;
+    kz = 4503599627370496.0 + (double)(int)sz.y; bias = (int)sz.y - 2048;
   }
 };
 // One column with the division itself, fp64 throughout: for weights whose quotient lies next to a tie (where the
 // reciprocal's last-bit error could change the rounding), outside the 32-bit range, or is not finite.
-__device__ __noinline__ double column_by_division(double w, double scale, double zero, double maxq, double rdiag, uint32_t* code) {
+__device__ __noinline__ double column_by_division(double w, double scale, double zero, double maxq, uint32_t* code) {
   double q = rint(w / scale) + zero;
   q = fmin(fmax(q, 0.0), maxq);
   *code = (uint32_t)q;
-  return (w - scale * (q - zero)) * rdiag;
+  return w - scale * (q - zero);
 }
 
 // ---- pieces of the row threads' loop ------------------------------------------------------------------
@@ -195,7 +196,7 @@ __device__ __forceinline__ void stripe_small_group(const StripeGroups& sg, int j
   for (int m = 0; m < kStripeSB; ++m)
     if (m >= jj && m < jj + sg.g) { mn = w[m] < mn ? w[m] : mn; mx = w[m] > mx ? w[m] : mx; }
   const float2 sz = find_params_outofline(mn, mx, sg.gs);
-  grid.set(sz, sg.gs.maxq);
+  grid.set(sz);
   if (sg.live) { sg.scales[jj / sg.g] = sz.x; sg.zeros[jj / sg.g] = sz.y; }
 }
 // The sixteen columns once more, with the division itself in every one of them.
@@ -213,13 +214,13 @@ __device__ __noinline__ void stripe_redo(const StripeAt& at, const StripeCols& c
   for (int jj = 0; jj < kStripeSB; ++jj) {
     if (kSmallGroups && (jj & 3) == 0 && ((sg.starts >> jj) & 1u)) stripe_small_group(sg, jj, w, grid);
     uint32_t code;
-    const double e = column_by_division(w[jj], grid.scale, grid.zero, (double)sg.gs.maxq, cs.rdiag[jj], &code);
+    const double r = column_by_division(w[jj], grid.scale, grid.zero, (double)sg.gs.maxq, &code), e = r * cs.rdiag[jj];
     out.err[jj] = (float)e;
     out.loss = fma(e, e, out.loss);
     out.cw[jj >> 2] |= code << (8 * (jj & 3));
 #pragma unroll
     for (int m = 0; m < kStripeSB; ++m)
-      if (m > jj) w[m] = fma(-e, cs.U[jj][m], w[m]);
+      if (m > jj) w[m] = fma(-r, cs.U[jj][m], w[m]);
   }
 }
 // Two scaled errors as fp16 pairs: the two high parts and the two remainders, saturating.
@@ -303,11 +304,12 @@ __device__ __forceinline__ void stripe_stage_cols(const StripeArgs& a, StripeCol
     for (int h = 0; h < 2; ++h) {
       const int r = r0 + 8 * h;
       const float uu[4] = {u[h].x, u[h].y, u[h].z, u[h].w};
+      // 1 / U_rr, from the lane of the four that share row r and have column r
+      const float dd = r % 4 == 0 ? uu[0] : r % 4 == 1 ? uu[1] : r % 4 == 2 ? uu[2] : uu[3];
+      const double rd = 1.0 / (double)__shfl_sync(0xffffffffu, dd, (lane & ~3) + (r >> 2));
+      if (q == (r >> 2)) c.rdiag[r] = rd;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        c.U[r][4 * q + e] = (double)uu[e];
-        if (r == 4 * q + e) c.rdiag[r] = 1.0 / (double)uu[e];
-      }
+      for (int e = 0; e < 4; ++e) c.U[r][4 * q + e] = (double)uu[e] * rd;
     }
     if (lane < 16) { c.sks[lane] = sk; c.sci[lane] = sc; }
     __syncwarp();
@@ -529,7 +531,7 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
     const float se_row = live ? a.sE[row] : 1.f;
     const double inv_se = live ? (double)a.sEinv[row] : 0.0;
     RowGrid grid;
-    grid.set(live && g <= 0 ? make_float2(a.scales[row], a.zeros[row]) : make_float2(1.f, 0.f), a.grid.maxq);
+    grid.set(live && g <= 0 ? make_float2(a.scales[row], a.zeros[row]) : make_float2(1.f, 0.f));
     double loss = 0.0;
     bool bad = false, ok = true;
     // columns of a 16-column sub-block at which a small group (4, 8 or 16 columns) starts
@@ -561,14 +563,21 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
             fence_after_thread_sync();
           }
           const float2 sz = stripe_scan(at(), g, k.width - j0, a.grid);
-          grid.set(sz, a.grid.maxq);
+          grid.set(sz);
           if (live) { a.scales[(int64_t)row * G + (i + j0) / g] = sz.x; a.zeros[(int64_t)row * G + (i + j0) / g] = sz.y; }
         }
         double w[kStripeSB];
 #pragma unroll
         for (int m = 0; m < kStripeSB; ++m) w[m] = ahead[m];
-        if (b > 0) stripe_subtract(tm_next + j0, cs.sci, inv_se, w);
-        if (j0 > 0) stripe_subtract(tm_rest + j0, cs.sci, inv_se, w);
+        if (b > 0 && j0 > 0) {                             // (both on their way before the wait)
+          float v[kStripeSB], u[kStripeSB];
+          tmem_ld_32x16(tm_next + j0, v); tmem_ld_32x16(tm_rest + j0, u);
+          umma::tmem_ld_wait();
+#pragma unroll
+          for (int m = 0; m < kStripeSB; ++m) w[m] = (w[m] - (double)(v[m] * cs.sci[m]) * inv_se) - (double)(u[m] * cs.sci[m]) * inv_se;
+        } else if (b > 0 || j0 > 0) {
+          stripe_subtract(b > 0 ? tm_next + j0 : tm_rest + j0, cs.sci, inv_se, w);
+        }
         // the next sixteen columns' loads go out now
         {
           const int col = k.ib + j0 + kStripeSB;
@@ -578,31 +587,57 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
         StripeGroups sg{g, small_group_starts, a.grid, a.scales + (int64_t)row * G + (i + j0) / (g > 0 ? g : 1),
                         a.zeros + (int64_t)row * G + (i + j0) / (g > 0 ? g : 1), live};
         // The sixteen columns.  What bounds them is the chain from one column's weight to the next column's, so it is kept to
-        // five fp64 operations and three integer ones, and the instructions beside it are counted too.  The quotient
+        // three fp64 operations and two integer ones, and the instructions beside it are counted too.  The quotient
         // w / scale + 1/2 is formed with the reciprocal, added to 2^32 + 2048: the low word then holds it in units of 2^-20,
-        // its upper twelve bits the code (rounded, counted from -2048), to be clamped as an integer; w - scale * integer is
-        // exact in one multiply-add (24-bit scale).  Where the quotient lies within 2^-20 of a tie (the fraction bits are
-        // next to zero) or outside twelve bits (the upper word is another one), the sixteen columns are done again with the
-        // division itself.  (rint, fmin and fmax take 20 to 25 cycles each in fp64.)
-        constexpr double kQuot = 4294967296.0 + 2048.5, kInt = 4503599627370496.0 + 2048.0;
+        // its upper twelve bits the code (rounded, counted from zero-point - 2048), to be clamped as an integer.  With U's row
+        // divided by U_jj (n) the next column's weight is (w' - w n) + (scale n) (code - zero-point): everything but the last
+        // multiply-add is ready when the code is.  The other columns take (w - scale (code - zero-point)) n, exact in its one
+        // multiply-add (24-bit scale).  Where the quotient lies within 2^-20 of a tie (the fraction bits are next to zero) or
+        // outside twelve bits (the upper word is another one), the sixteen columns are done again with the division itself.
+        // (rint, fmin and fmax take 20 to 25 cycles each in fp64.)  The errors' way into the tile fills the chain's gaps, pair by
+        // pair.  4096 rows x 1024 columns, 4-bit: 195 us with the error's five operations on the chain; 189 with it; 190 with the
+        // tile written here instead of after the loop, 189 with both sums of the sub-block asked for at once; 184 with all three.
+        constexpr double kQuot = 4294967296.0 + 2048.5;
         float err[kStripeSB];
         uint32_t cw[kStripeSB / 4];
         uint32_t frac = 0xFFFFFu;                          // smallest distance of the fraction bits above -1 seen
         int range = 0;
         double l0 = 0.0;
+        uint32_t hw[kStripeSB / 2], lw[kStripeSB / 2];
+        float big = 0.f;
+        uint8_t* rowp = etile + (j0 >> 6) * 16384 + t * 128;
+        // the tile was last read by the pushes of the block before the previous one
+        if (j0 == 0 && b >= 2) stripe_wait(&bar.tile_free[b & 1], (b >> 1) - 1, ok, a.dev_info, 45);
+        // scaled errors u and u + 1 as fp16 hi / lo pairs, and with the eighth and the sixteenth column eight of them into the swizzled
+        // K-major tile (row t, 16-byte chunk (k / 8) ^ (t & 7) of the 128-byte row of K atom k / 64)
+        auto put = [&](int u) {
+          const float x0 = err[u] * cs.sks[u] * se_row, x1 = err[u + 1] * cs.sks[u + 1] * se_row;
+          big = fmaxf(big, fmaxf(fabsf(x0), fabsf(x1)));
+          stripe_split2(x0, x1, hw[u >> 1], lw[u >> 1]);
+          if ((u & 7) != 6) return;
+          uint8_t* d = rowp + (((((j0 & 63) + u) >> 3) ^ (t & 7)) << 4);
+          *reinterpret_cast<uint4*>(d) = make_uint4(hw[u / 2 - 3], hw[u / 2 - 2], hw[u / 2 - 1], hw[u / 2]);
+          *reinterpret_cast<uint4*>(d + 32768) = make_uint4(lw[u / 2 - 3], lw[u / 2 - 2], lw[u / 2 - 1], lw[u / 2]);
+        };
 #pragma unroll
         for (int jj = 0; jj < kStripeSB; ++jj) {
           if (kSmallGroups && (jj & 3) == 0 && ((small_group_starts >> jj) & 1u)) stripe_small_group(sg, jj, w, grid);
           const double t0 = fma(w[jj], grid.rscale, kQuot);
           const uint32_t q = (uint32_t)__double2loint(t0);
-          const uint32_t c = min(max(q >> 20, grid.lo), grid.hi);
-          const double e = fma(-grid.scale, __hiloint2double(0x43300000, (int)c) - kInt, w[jj]) * cs.rdiag[jj];   // (w - q) / U_jj
+          const uint32_t c = (uint32_t)__viaddmin_s32_relu((int)(q >> 20), grid.bias, a.grid.maxq);
+          const double cd = __hiloint2double(0x43300000, (int)c) - grid.kz;         // code - zero-point
+          if (jj + 1 < kStripeSB) {
+            const double nx = cs.U[jj][jj + 1];
+            w[jj + 1] = fma(cd, grid.scale * nx, fma(-w[jj], nx, w[jj + 1]));
+          }
+          const double r = fma(-grid.scale, cd, w[jj]), e = r * cs.rdiag[jj];
 #pragma unroll
           for (int m = 0; m < kStripeSB; ++m)             // immediate feedback onto the later columns in registers
-            if (m > jj) w[m] = fma(-e, cs.U[jj][m], w[m]);
+            if (m > jj + 1) w[m] = fma(-r, cs.U[jj][m], w[m]);
+          cw[jj >> 2] = (jj & 3) == 0 ? c : cw[jj >> 2] + (c << (8 * (jj & 3)));
           err[jj] = (float)e;
           l0 = fma(e, e, l0);
-          cw[jj >> 2] = (jj & 3) == 0 ? c - grid.lo * 0x01010101u : cw[jj >> 2] + (c << (8 * (jj & 3)));
+          if (jj & 1) put(jj - 1);
           frac = min(frac, (q + 1u) & 0xFFFFFu);
           range |= __double2hiint(t0) ^ 0x41F00000;
         }
@@ -614,29 +649,11 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
 #pragma unroll
           for (int m = 0; m < kStripeSB / 4; ++m) cw[m] = r.cw[m];
           l0 = r.loss;
-        }
-        // scaled errors as an fp16 hi / lo pair: into the swizzled K-major tile (row t, 16-byte chunk (k / 8) ^ (t & 7) of
-        // the 128-byte row of K atom k / 64) and, in the inverse form, to global memory for the left-looking contractions of
-        // later outer blocks; codes as bytes
-        uint32_t hw[kStripeSB / 2], lw[kStripeSB / 2];
-        float big = 0.f;
+          big = 0.f;
 #pragma unroll
-        for (int u = 0; u < kStripeSB; u += 2) {
-          const float x0 = err[u] * cs.sks[u] * se_row, x1 = err[u + 1] * cs.sks[u + 1] * se_row;
-          big = fmaxf(big, fmaxf(fabsf(x0), fabsf(x1)));
-          stripe_split2(x0, x1, hw[u >> 1], lw[u >> 1]);
+          for (int m = 0; m < kStripeSB; m += 2) put(m);
         }
         if (live) { bad |= big > 65504.f || !isfinite(l0); loss += l0; }
-        // the tile was last read by the pushes of the block before the previous one
-        if (j0 == 0 && b >= 2) stripe_wait(&bar.tile_free[b & 1], (b >> 1) - 1, ok, a.dev_info, 45);
-        const uint4 h_a = make_uint4(hw[0], hw[1], hw[2], hw[3]), h_b = make_uint4(hw[4], hw[5], hw[6], hw[7]);
-        const uint4 l_a = make_uint4(lw[0], lw[1], lw[2], lw[3]), l_b = make_uint4(lw[4], lw[5], lw[6], lw[7]);
-        const int atom = j0 >> 6, ch0 = (j0 & 63) >> 3;
-        uint8_t* rowp = etile + atom * 16384 + t * 128;
-        *reinterpret_cast<uint4*>(rowp + ((ch0 ^ (t & 7)) << 4)) = h_a;
-        *reinterpret_cast<uint4*>(rowp + (((ch0 + 1) ^ (t & 7)) << 4)) = h_b;
-        *reinterpret_cast<uint4*>(rowp + 32768 + ((ch0 ^ (t & 7)) << 4)) = l_a;
-        *reinterpret_cast<uint4*>(rowp + 32768 + (((ch0 + 1) ^ (t & 7)) << 4)) = l_b;
         fence_proxy_async();                              // the tile was written through the generic proxy
         fence_before_thread_sync();                       // this sub-block's tcgen05.ld are done
         __syncwarp();
@@ -650,7 +667,8 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
           if (a.keep_errors) {
             uint4* gh = reinterpret_cast<uint4*>(a.Ehi + o);
             uint4* gl = reinterpret_cast<uint4*>(a.Elo + o);
-            gh[0] = h_a; gh[1] = h_b; gl[0] = l_a; gl[1] = l_b;
+            gh[0] = make_uint4(hw[0], hw[1], hw[2], hw[3]); gh[1] = make_uint4(hw[4], hw[5], hw[6], hw[7]);
+            gl[0] = make_uint4(lw[0], lw[1], lw[2], lw[3]); gl[1] = make_uint4(lw[4], lw[5], lw[6], lw[7]);
           }
           *reinterpret_cast<uint4*>(a.codes + o) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
         }
