@@ -1102,3 +1102,24 @@ def test_dequantize_at_the_edges_of_a_thread(B, bits, R, C, group, off):
     s, z = np.repeat(scales, C // G, 1), np.repeat(zeros, C // G, 1)
     want = (s * (codes.astype(np.float32) - z)).astype(np.float16)
     assert np.array_equal(out.cpu().numpy().view(np.uint16), want.view(np.uint16))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 8])
+@pytest.mark.parametrize("R,C", [(1, 32), (3, 96), (65, 288)])
+def test_packed_words_wherever_they_go(B, bits, R, C):
+    """The packing kernel takes 32 codes per thread and stores 16 bytes at a time where the output allows: the same words 4 bytes off."""
+    W = torch.from_numpy(_layer(R, C, 64, cfg=16).w()).cuda()
+    U = torch.eye(C, device="cuda")
+    ref = B.gptq_quantize_layer(W, U, bits, 0, False, 32)
+    words = torch.zeros(ref["qweight"].numel() + 4, dtype=torch.int32, device="cuda")
+    for off in (0, 1, 2):
+        q = words[off:off + ref["qweight"].numel()].view_as(ref["qweight"])
+        ws = torch.empty(B.gptq_quantize_workspace_bytes(R, C, bits, 0, 32), dtype=torch.uint8, device="cuda")
+        info, loss = torch.zeros(2, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.float64, device="cuda")
+        sc, ze = torch.empty_like(ref["scales"]), torch.empty_like(ref["zeros"])
+        st = B._lib.gptq_quantize_layer(W.data_ptr(), U.data_ptr(), R, C, bits, 0, 0, 32, q.data_ptr(), sc.data_ptr(), ze.data_ptr(),
+                                        loss.data_ptr(), ws.data_ptr(), ws.numel(), info.data_ptr(), B._stream_ptr(None))
+        torch.cuda.synchronize()
+        assert st == B.OK and torch.equal(q, ref["qweight"])
+    codes, _ = O.rtn(W.cpu().numpy(), bits, 0, False)                          # (no feedback: U is the identity)
+    assert np.array_equal(O.pack_codes(codes, bits), ref["qweight"].cpu().numpy().view(np.uint32))
