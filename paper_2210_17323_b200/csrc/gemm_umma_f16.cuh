@@ -87,6 +87,11 @@ struct TileItems {
   }
 };
 
+// Epilogues that add to what is there (kAccumulates; those that leave through TMA reductions all do): a tile's K may be cut as fine
+// as it pays.  The others get the whole K in one item.
+template <class T, class = void> struct accumulates { static constexpr bool value = pipe2::is_tile_epilogue<T>::value; };
+template <class T> struct accumulates<T, decltype((void)T::kAccumulates)> { static constexpr bool value = true; };
+
 // Host-side description of one operand pair (hi, lo share the geometry).
 struct Operand {
   const __half* hi; const __half* lo;
@@ -113,6 +118,12 @@ gptq_status_t launch(const Operand& A, const Operand& B, int M, int N, EpiF epi,
   if ((st = mk(&maps.b_hi, B.hi, B)) != GPTQ_OK) return st;
   if ((st = mk(&maps.b_lo, B.lo, B)) != GPTQ_OK) return st;
   TileItems<kTriLeft, kUpperOut> items{(M + BM - 1) / BM, (N + BN - 1) / BN, (int)((K + BK - 1) / BK), kSuperK / BK};
+  if (accumulates<EpiF>::value) {
+    // Few tiles (a 1024-column block of a narrow layer, a diagonal block of the factor): K is cut until every CTA pair has an item, but
+    // not below 512, where an item's sums take as long to leave as to make.
+    const int tiles = kUpperOut ? items.tiles_m * (items.tiles_m + 1) / 2 : items.tiles_m * items.tiles_n, pairs = (device_sm_count() - reserve_sms) / 2;
+    while (items.sc_kb > 8 && tiles * ((items.kb_total + items.sc_kb - 1) / items.sc_kb) < pairs) items.sc_kb /= 2;
+  }
   const int n_sc = (items.kb_total + items.sc_kb - 1) / items.sc_kb;
   return pipe2::launch_pipe2<Traits>(maps, (int64_t)items.tiles_m * items.tiles_n * n_sc, items, epi, dev_info, stream,
                                      reserve_sms);

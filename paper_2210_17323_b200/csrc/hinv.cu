@@ -108,6 +108,7 @@ __global__ void inverse_row_scales_kernel(const float* __restrict__ U, int C, co
 // Every epilogue multiplies the partial sum by sa[row] * sb[col] (powers of two: the operands' scalings undone).
 // dst[row][cofs + col] -= partial for elements on or above the diagonal (fp32 reductions).
 struct EpiSubUpperRed {
+  static constexpr bool kAccumulates = true;
   float* p; int64_t ld; int cofs; int M, N;
   const float* sa; const float* sb;
   __device__ __forceinline__ void operator()(int row, int col0, const float (&v)[32]) const {

@@ -522,6 +522,7 @@ __global__ void residual_pair_kernel(const __half* __restrict__ W, const uint8_t
 // Wblk[row][nofs + col ..) -= partial / (sE[row] sC[column]), as fp64 reductions: partial sums of one tile
 // come from several CTA pairs (one per super-chunk of the contraction).
 struct EpiSubWblk {
+  static constexpr bool kAccumulates = true;
   double* Wblk; int64_t ldw; int nofs; int R, N;
   const float* sEinv; const float* sCinv;     // sCinv already offset to the first column of this contraction
   int stripe_major;                           // layout of Wblk (see wblk_from_w16_kernel)
