@@ -277,7 +277,17 @@ gptq_status_t hessian_umma(float* H, const __nv_bfloat16* X, int64_t n_tokens, i
     it.wt = 144;
     it.n_enum = it.tiles * (it.tiles + 1) / 2;
     ck = 128;                             // 8192 tokens per item
-    while (ck > 8 && (int64_t)it.n_enum * ceil_div(total_kb, ck) < sms) ck >>= 1;
+    // Few items: what counts is full rounds of the CTA pairs, and that an item's sums take as long to leave as 13 of its token blocks
+    // to add up (5 us).  The cheapest number of equal token ranges per tile, by rounds x (blocks + 13).
+    const int pairs = sms / 2 > 0 ? sms / 2 : 1;
+    if ((int64_t)it.n_enum * ceil_div(total_kb, ck) < 6 * (int64_t)pairs) {
+      int64_t best = -1;
+      for (int n = ceil_div(total_kb, 128); n <= ceil_div(total_kb, 4) && n <= 64; ++n) {
+        const int per = ceil_div(total_kb, n);
+        const int64_t cost = (int64_t)ceil_div((int64_t)it.n_enum * ceil_div(total_kb, per), pairs) * (per + 13);
+        if (best < 0 || cost < best) { best = cost; ck = per; }
+      }
+    }
     while ((int64_t)it.n_enum * ceil_div(total_kb, ck) > 0x3FFFFFFF) ck <<= 1;     // (the grid has one cluster per item)
     it.total_kb = total_kb; it.sc_kb = ck; it.nsc = ceil_div(total_kb, ck);
     const int64_t n_items = (int64_t)it.n_enum * it.nsc;

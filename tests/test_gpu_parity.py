@@ -1123,3 +1123,18 @@ def test_packed_words_wherever_they_go(B, bits, R, C):
         assert st == B.OK and torch.equal(q, ref["qweight"])
     codes, _ = O.rtn(W.cpu().numpy(), bits, 0, False)                          # (no feedback: U is the identity)
     assert np.array_equal(O.pack_codes(codes, bits), ref["qweight"].cpu().numpy().view(np.uint32))
+
+
+@pytest.mark.parametrize("C,tokens", [(512, 1), (512, 64), (512, 65), (544, 1000), (768, 8192), (2400, 5001), (1024, 20000)])
+def test_hessian_however_its_tokens_are_cut(B, C, tokens):
+    """Token ranges per tile are chosen by rounds of the CTA pairs; whole-number activations whose sums stay below 2^24 give the same
+    Hessian, exactly, however they are cut."""
+    g = torch.Generator("cuda").manual_seed(C + tokens)
+    X = torch.randint(-2, 3, (tokens, C), device="cuda", generator=g).to(torch.bfloat16)
+    H = torch.zeros((C, C), device="cuda")
+    B.gptq_hessian_accumulate(H, X)
+    want = torch.zeros((C, C), dtype=torch.float64, device="cuda")
+    for t in range(0, tokens, 4096):
+        x = X[t:t + 4096].double()
+        want += 2 * x.T @ x
+    assert torch.equal(H.double(), want)
