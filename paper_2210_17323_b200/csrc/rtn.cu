@@ -2,7 +2,7 @@
 // exactly the grid the solver would use for untouched weights -- per-row or per-group min-max,
 // asymmetric with an integer zero-point (or symmetric / ternary) -- with no error feedback.
 // Output layout is that of gptq_quantize_layer.  One pass over W for groups that are multiples of 32 columns and per-row
-// grids (rtn_span_kernel, rtn_fused_kernel), two plain passes for the small groups (4, 8, 16).
+// grids (rtn_span_kernel, rtn_held_kernel), two plain passes for the small groups (4, 8, 16).
 #include "common.cuh"
 
 namespace gptq {
@@ -70,10 +70,9 @@ __global__ void rtn_pack_kernel(const __half* __restrict__ W, int R, int C, int 
 
 // ---- one pass for groups that are multiples of 32 columns (and per-row grids) -----------------------------------
 // Groups are bound by issue slots (78 % of them filled, 20 instructions a weight with what carries minima and grids between
-// lanes), per-row grids by the latency of their loads and by W's second read, half of which misses L2 (11 instructions a
-// weight, 50 % of the slots).  So: one instruction a weight for the minimum and maximum (half2), few for the code, four loads
-// in flight.  (12288 x 12288, 4-bit per row: 178 us with single-precision minima, a branch per code and one load in flight
-// in the second pass; 113 now, where the bytes alone take 57.)
+// lanes); wider ones by the latency of their loads and what each row waits for between them (rtn_held_kernel).  So: one instruction
+// a weight for the minimum and maximum (half2), few for the code, several loads in flight.  (12288 x 12288, 4-bit per row: 178 us
+// with single-precision minima, a branch per code and one load in flight in the second pass, where the bytes alone take 57.)
 __device__ __forceinline__ void rtn_grid_of(float mn, float mx, RtnGrid grid, float& scale, float& zero) {
   double xmin = fmin((double)mn, 0.0), xmax = fmax((double)mx, 0.0);
   if (xmin == 0.0 && xmax == 0.0) { xmin = -1.0; xmax = 1.0; }
@@ -176,9 +175,77 @@ __device__ __forceinline__ void rtn_store_words(uint32_t* qrow, int i, bool on, 
   }
 }
 
-// One warp per (row, group), any group that is a multiple of 32 columns.  Phase A: the group's minimum and maximum from
-// 16-byte loads (a lane takes the 8-column pieces lane, lane + 32, ...).  Phase B: the same pieces again (now from L1 /
-// L2: the group was just read), eight codes per lane, stored as whole words.  W comes from memory once.
+// kThreads threads per (row, group) with at most kHeld pieces of 8 columns each: a thread loads its pieces (t, t + kThreads, ...) all at
+// once and keeps them in registers, the group's minimum and maximum go through the warps and, if there are several, through shared
+// memory, one thread derives the grid, and the codes are made from the registers.  W is read once.  (One warp per row that read W again
+// for the codes, half of it from DRAM: 114 us for 12288 x 12288, 4-bit; this form 105; a ring in shared memory that asynchronous copies fill
+// one row ahead: 121.)  Groups of up to 2048 columns go to a warp, eight of them to a CTA, wider ones to a CTA of 128 to 1024 threads.
+template <int F, int kThreads, int kHeld>
+__global__ void __launch_bounds__(kThreads == 32 ? 256 : kThreads)
+rtn_held_kernel(const __half* __restrict__ W, int R, int C, int g, int G, RtnGrid grid,
+                float* __restrict__ scales, float* __restrict__ zeros, uint32_t* __restrict__ qweight) {
+  __shared__ float red[kThreads / 32][2], made[2];
+  const int lane = threadIdx.x & 31, t = kThreads == 32 ? lane : threadIdx.x, warp = threadIdx.x >> 5;
+  const int64_t wid = kThreads == 32 ? (int64_t)blockIdx.x * (blockDim.x >> 5) + warp : (int64_t)blockIdx.x;
+  if (wid >= (int64_t)R * G) return;                        // (a whole warp; with more threads per group there is none)
+  const int row = (int)(wid / G), gi = (int)(wid % G);
+  const uint4* p = reinterpret_cast<const uint4*>(W + (int64_t)row * C + (int64_t)gi * g);
+  const int pieces = g / 8;
+  uint4 v[kHeld];
+#pragma unroll
+  for (int u = 0; u < kHeld; ++u)
+    if (t + kThreads * u < pieces) v[u] = __ldcs(p + t + kThreads * u);
+  __half2 mn = rtn_half2_const(0x7C00), mx = rtn_half2_const(0xFC00);        // +inf, -inf
+#pragma unroll
+  for (int u = 0; u < kHeld; ++u)
+    if (t + kThreads * u < pieces) rtn_minmax8(v[u], mn, mx);
+  for (int o = 16; o > 0; o >>= 1) { mn = rtn_reduce_step<true>(mn, o); mx = rtn_reduce_step<false>(mx, o); }
+  float lo = rtn_low(mn), hi = rtn_high(mx);                // (the same in every lane)
+  if constexpr (kThreads > 32) {
+    if (lane == 0) { red[warp][0] = lo; red[warp][1] = hi; }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) {               // (a NaN is kept)
+      const float h = red[w][1];
+      lo = fminf(lo, red[w][0]);
+      hi = isnan(hi) ? hi : isnan(h) ? h : fmaxf(hi, h);
+    }
+  }
+  const bool finite = rtn_finite(lo, hi);
+  if (isnan(hi)) {                                          // (the same in every thread)
+    hi = rtn_high_of_numbers(p, lane, pieces, 32);
+    for (int o = 16; o > 0; o >>= 1) hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  float scale = 0.f, zero = 0.f;
+  if (t == 0) {
+    rtn_grid_of(lo, hi, grid, scale, zero);
+    scales[wid] = scale; zeros[wid] = zero;
+    if (kThreads > 32) { made[0] = scale; made[1] = zero; }
+  }
+  if constexpr (kThreads > 32) {
+    __syncthreads();
+    scale = made[0]; zero = made[1];
+  } else {
+    scale = __shfl_sync(0xffffffffu, scale, 0);
+    zero = __shfl_sync(0xffffffffu, zero, 0);
+  }
+  const float rs = finite ? 1.0f / scale : 0.f;
+  // words of this group inside the row: the group starts at bit gi * g * F, a multiple of 32 F bits
+  uint32_t* qrow = qweight + (int64_t)row * (C / 32 * F) + (int64_t)gi * (g / 32 * F);
+#pragma unroll
+  for (int u = 0; u < kHeld; ++u) {
+    if (kThreads * u >= pieces) break;                      // (uniform: every lane of a warp joins the shuffles)
+    const int i = t + kThreads * u;
+    const bool on = i < pieces;
+    uint64_t bits = 0;
+    if (on) bits = rtn_codes8<F>(v[u], scale, rs, zero, grid.maxq);
+    rtn_store_words<F>(qrow, i, on, bits, lane);
+  }
+}
+
+// One warp per (row, group) for groups that are too wide for that (beyond 65536 columns).  Phase A: the group's minimum and
+// maximum from 16-byte loads (a lane takes the 8-column pieces lane, lane + 32, ...).  Phase B: the same pieces again, eight codes
+// per lane, stored as whole words.
 template <int F>
 __global__ void __launch_bounds__(256)
 rtn_fused_kernel(const __half* __restrict__ W, int R, int C, int g, int G, RtnGrid grid,
@@ -309,12 +376,16 @@ extern "C" gptq_status_t gptq_rtn_layer(const void* W_fp16, int R, int C, int bi
   if (g % 32 == 0 && aligned_to(W_fp16, 16)) {              // one pass; (row, group) starts are then 16-byte aligned too
     const bool span = g == 32 || g == 64 || g == 128 || g == 256;
     const int64_t warps = span ? (int64_t)R * ((G + 31) / 32) : (int64_t)R * G;
-    const unsigned blocks = (unsigned)((warps + 7) / 8);
+    const unsigned blocks = (unsigned)((warps + 7) / 8), groups = (unsigned)((int64_t)R * G);
 #define GPTQ_RTN_LAUNCH(FF)                                                                                               \
     if (g == 32) rtn_span_kernel<FF, 4><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);                 \
     else if (g == 64) rtn_span_kernel<FF, 8><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);            \
     else if (g == 128) rtn_span_kernel<FF, 16><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);          \
     else if (g == 256) rtn_span_kernel<FF, 32><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);          \
+    else if (g <= 2048) rtn_held_kernel<FF, 32, 8><<<blocks, 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);            \
+    else if (g <= 8192) rtn_held_kernel<FF, 128, 8><<<groups, 128, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);        \
+    else if (g <= 16384) rtn_held_kernel<FF, 256, 8><<<groups, 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);        \
+    else if (g <= 65536) rtn_held_kernel<FF, 1024, 8><<<groups, 1024, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);        \
     else rtn_fused_kernel<FF><<<blocks, 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight)
     switch (f) {
       case 2: GPTQ_RTN_LAUNCH(2); break;

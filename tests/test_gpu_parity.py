@@ -1138,3 +1138,18 @@ def test_hessian_however_its_tokens_are_cut(B, C, tokens):
         x = X[t:t + 4096].double()
         want += 2 * x.T @ x
     assert torch.equal(H.double(), want)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 8])
+@pytest.mark.parametrize("R,C,group", [(3, 288, 288), (5, 2048, 0), (700, 2080, 0), (1300, 2080, 0), (9, 4608, 2304), (2, 16416, 0), (2, 65536, 0), (2, 65568, 0)])
+def test_rtn_of_wide_groups(B, bits, R, C, group):
+    """Groups of up to 2048 columns stay in a warp's registers, wider ones in those of a CTA of more and more threads, and those beyond
+    65536 columns are read twice: sizes at the edges of each."""
+    W16 = (0.02 * np.random.default_rng(C + bits).standard_normal((R, C))).astype(np.float16)
+    out = B.gptq_rtn_layer(torch.from_numpy(W16).cuda(), bits, group, False)
+    codes, _ = O.rtn(W16, bits, group, False)
+    assert np.array_equal(O.pack_codes(codes, bits), out["qweight"].cpu().numpy().view(np.uint32))
+    g = group if group > 0 else C
+    grids = [O.find_params(W16[:, j:j + g].astype(np.float64), bits, False) for j in range(0, C, g)]
+    assert np.array_equal(out["scales"].cpu().numpy().astype(np.float64), np.stack([a for a, _ in grids], 1))
+    assert np.array_equal(out["zeros"].cpu().numpy().astype(np.float64), np.stack([b for _, b in grids], 1))
