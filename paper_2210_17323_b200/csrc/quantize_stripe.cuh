@@ -298,7 +298,7 @@ __device__ __forceinline__ void stripe_stage_cols(const StripeArgs& a, StripeCol
   fetch(0);
   bool ok = true;
   for (int n = 0; n < n_sub; ++n) {
-    if (!stripe_wait(&bar.cols_empty[n & 1], (n >> 1) ^ 1, ok, a.dev_info, 38)) return;
+    if (!__all_sync(0xffffffffu, stripe_wait(&bar.cols_empty[n & 1], (n >> 1) ^ 1, ok, a.dev_info, 38))) return;   // (they shuffle below)
     StripeCols& c = cols[n & 1];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
