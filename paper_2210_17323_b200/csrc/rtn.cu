@@ -2,7 +2,7 @@
 // exactly the grid the solver would use for untouched weights -- per-row or per-group min-max,
 // asymmetric with an integer zero-point (or symmetric / ternary) -- with no error feedback.
 // Output layout is that of gptq_quantize_layer.  One pass over W for groups that are multiples of 32 columns and per-row
-// grids (rtn_span_kernel, rtn_held_kernel), two plain passes for the small groups (4, 8, 16).
+// grids (rtn_span_kernel, rtn_held_kernel, rtn_fused_kernel), two plain passes for the small groups (4, 8, 16).
 #include "common.cuh"
 
 namespace gptq {
@@ -177,11 +177,14 @@ __device__ __forceinline__ void rtn_store_words(uint32_t* qrow, int i, bool on, 
 
 // kThreads threads per (row, group) with at most kHeld pieces of 8 columns each: a thread loads its pieces (t, t + kThreads, ...) all at
 // once and keeps them in registers, the group's minimum and maximum go through the warps and, if there are several, through shared
-// memory, one thread derives the grid, and the codes are made from the registers.  W is read once.  (One warp per row that read W again
-// for the codes, half of it from DRAM: 114 us for 12288 x 12288, 4-bit; this form 105; a ring in shared memory that asynchronous copies fill
-// one row ahead: 121.)  Groups of up to 2048 columns go to a warp, eight of them to a CTA, wider ones to a CTA of 128 to 1024 threads.
+// memory, one thread derives the grid, and the codes are made from the registers.  W is read once.  One warp per group, eight of them to
+// a CTA, or a CTA per group.  A group's load, minimum, grid and codes follow one another, so what counts is how many bytes of W an SM has
+// on their way: the pieces fill the threads (kHeld and kThreads follow the group's width, see rtn_launch) and the minimum of CTAs per SM keeps a
+// thread at 64 registers, 80 where a warp holds 6 or 8 (512 threads, 32768 columns: 2 CTAs an SM instead of 1, 107 instead of 154 us for 1.5e8 weights).
+// 12288 x 12288, 4-bit: 90 us, where the bytes alone take 57 (192 threads; with 256 of them a quarter idle 103; rtn_fused_kernel, which reads W
+// twice, half of it from DRAM: 112; a ring in shared memory that asynchronous copies fill one row ahead: 121).
 template <int F, int kThreads, int kHeld>
-__global__ void __launch_bounds__(kThreads == 32 ? 256 : kThreads)
+__global__ void __launch_bounds__(kThreads == 32 ? 256 : kThreads, kThreads == 32 ? (kHeld <= 4 ? 4 : 3) : 1024 / kThreads)
 rtn_held_kernel(const __half* __restrict__ W, int R, int C, int g, int G, RtnGrid grid,
                 float* __restrict__ scales, float* __restrict__ zeros, uint32_t* __restrict__ qweight) {
   __shared__ float red[kThreads / 32][2], made[2];
@@ -243,9 +246,10 @@ rtn_held_kernel(const __half* __restrict__ W, int R, int C, int g, int G, RtnGri
   }
 }
 
-// One warp per (row, group) for groups that are too wide for that (beyond 65536 columns).  Phase A: the group's minimum and
-// maximum from 16-byte loads (a lane takes the 8-column pieces lane, lane + 32, ...).  Phase B: the same pieces again, eight codes
-// per lane, stored as whole words.
+// One warp per (row, group), any group that is a multiple of 32 columns.  Phase A: the group's minimum and maximum from 16-byte loads (a
+// lane takes the 8-column pieces lane, lane + 32, ...).  Phase B: the same pieces again, eight codes per lane, stored as whole words.
+// Nothing waits for another warp, and 32 rows an SM are in flight: the faster form where there are many groups of a width that fills the
+// threads of the form above badly, and the only one beyond 65536 columns.
 template <int F>
 __global__ void __launch_bounds__(256)
 rtn_fused_kernel(const __half* __restrict__ W, int R, int C, int g, int G, RtnGrid grid,
@@ -357,6 +361,42 @@ rtn_span_kernel(const __half* __restrict__ W, int R, int C, int G, RtnGrid grid,
   }
 }
 
+// Which form a group of g columns gets.  A warp's 32 lanes hold 4, 6 or 8 pieces each, a CTA's threads 8.  Where W is large and the group
+// has fewer columns than its form's `least`, rtn_fused_kernel: it needs a few waves of rows to get going (below 1e8 weights the forms that
+// hold a group win or tie at every width: 8000 rows of 4096 columns 24 against 26 us, of 10240 57 against 69), and from there on its time per weight
+// hardly depends on the width; beyond 2.5e8 weights it is the faster one up to 8192 columns.  Few groups leave SMs idle, so a group gets the
+// next wider CTA there (300 rows: 3072 columns on 64 / 128 threads 7.8 / 6.2 us, 12288 on 192 / 256 10.3 / 8.3).  Both sides, 4-bit, held / fused, 1.5e8 weights:
+// 288 columns 281 / 330 us, 1024 113 / 117, 1536 99 / 125, 1920 102 / 130, 2048 101 / 97, 2560 101 / 108, 3072 94 / 93, 4096 86 / 85, 5120 92 / 87, 6144 88 / 92,
+// 8192 89 / 94, 9216 102 / 98, 10240 97 / 101, 11264 95 / 109, 12288 90 / 112, 16384 92 / 124, 18432 125 / 130, 24576 111 / 141, 32768 107 / 146,
+// 36864 160 / 151, 40960 152 / 145 (8-bit 183 / 223: the 768 threads are kept), 49152 140 / 159, 65536 135 / 170;
+// 3e8 weights: 4096 163 / 156, 8192 166 / 159, 10240 185 / 170, 12288 172 / 187, 20480 232 / 230, 24576 214 / 236, 40960 296 / 261, 65536 259 / 279.
+template <int F>
+void rtn_launch(const __half* W, int R, int C, int g, int G, RtnGrid grid, float* scales, float* zeros, uint32_t* qweight, cudaStream_t s) {
+  const int64_t groups = (int64_t)R * G, runs = (int64_t)R * ((G + 31) / 32);
+  const auto warps = [](int64_t n) { return (unsigned)((n + 7) / 8); };
+  if (g == 32) { rtn_span_kernel<F, 4><<<warps(runs), 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight); return; }
+  if (g == 64) { rtn_span_kernel<F, 8><<<warps(runs), 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight); return; }
+  if (g == 128) { rtn_span_kernel<F, 16><<<warps(runs), 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight); return; }
+  if (g == 256) { rtn_span_kernel<F, 32><<<warps(runs), 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight); return; }
+  using Kernel = void (*)(const __half*, int, int, int, int, RtnGrid, float*, float*, uint32_t*);
+  struct Form { int widest, least, threads; Kernel kernel; };    // (least 2049: no group of 2048 columns where W is large)
+  static const Form forms[] = {
+      {1024, 0, 32, rtn_held_kernel<F, 32, 4>},      {1536, 0, 32, rtn_held_kernel<F, 32, 6>},      {2016, 0, 32, rtn_held_kernel<F, 32, 8>},
+      {2048, 2049, 32, rtn_held_kernel<F, 32, 8>},   {4096, 3328, 64, rtn_held_kernel<F, 64, 8>},   {6144, 5632, 96, rtn_held_kernel<F, 96, 8>},
+      {8192, 6656, 128, rtn_held_kernel<F, 128, 8>}, {12288, 11264, 192, rtn_held_kernel<F, 192, 8>}, {16384, 0, 256, rtn_held_kernel<F, 256, 8>},
+      {24576, 22528, 384, rtn_held_kernel<F, 384, 8>}, {32768, 0, 512, rtn_held_kernel<F, 512, 8>}, {49152, F == 8 ? 0 : 45056, 768, rtn_held_kernel<F, 768, 8>},
+      {65536, 0, 1024, rtn_held_kernel<F, 1024, 8>}};
+  const int64_t weights = groups * g;
+  for (const Form& form : forms) {
+    if (g > form.widest || (groups <= 1024 && (form.threads == 64 || form.threads == 96 || form.threads == 192))) continue;
+    if ((g < form.least && weights > 100000000) || (g >= 2048 && g <= 8192 && weights > 250000000)) break;
+    if (form.threads == 32) form.kernel<<<warps(groups), 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);
+    else form.kernel<<<(unsigned)groups, form.threads, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);
+    return;
+  }
+  rtn_fused_kernel<F><<<warps(groups), 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);
+}
+
 }  // namespace
 }  // namespace gptq
 
@@ -374,26 +414,12 @@ extern "C" gptq_status_t gptq_rtn_layer(const void* W_fp16, int R, int C, int bi
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __half* W = static_cast<const __half*>(W_fp16);
   if (g % 32 == 0 && aligned_to(W_fp16, 16)) {              // one pass; (row, group) starts are then 16-byte aligned too
-    const bool span = g == 32 || g == 64 || g == 128 || g == 256;
-    const int64_t warps = span ? (int64_t)R * ((G + 31) / 32) : (int64_t)R * G;
-    const unsigned blocks = (unsigned)((warps + 7) / 8), groups = (unsigned)((int64_t)R * G);
-#define GPTQ_RTN_LAUNCH(FF)                                                                                               \
-    if (g == 32) rtn_span_kernel<FF, 4><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);                 \
-    else if (g == 64) rtn_span_kernel<FF, 8><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);            \
-    else if (g == 128) rtn_span_kernel<FF, 16><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);          \
-    else if (g == 256) rtn_span_kernel<FF, 32><<<blocks, 256, 0, s>>>(W, R, C, G, grid, scales, zeros, qweight);          \
-    else if (g <= 2048) rtn_held_kernel<FF, 32, 8><<<blocks, 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);            \
-    else if (g <= 8192) rtn_held_kernel<FF, 128, 8><<<groups, 128, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);        \
-    else if (g <= 16384) rtn_held_kernel<FF, 256, 8><<<groups, 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);        \
-    else if (g <= 65536) rtn_held_kernel<FF, 1024, 8><<<groups, 1024, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight);        \
-    else rtn_fused_kernel<FF><<<blocks, 256, 0, s>>>(W, R, C, g, G, grid, scales, zeros, qweight)
     switch (f) {
-      case 2: GPTQ_RTN_LAUNCH(2); break;
-      case 3: GPTQ_RTN_LAUNCH(3); break;
-      case 4: GPTQ_RTN_LAUNCH(4); break;
-      default: GPTQ_RTN_LAUNCH(8); break;
+      case 2: rtn_launch<2>(W, R, C, g, G, grid, scales, zeros, qweight, s); break;
+      case 3: rtn_launch<3>(W, R, C, g, G, grid, scales, zeros, qweight, s); break;
+      case 4: rtn_launch<4>(W, R, C, g, G, grid, scales, zeros, qweight, s); break;
+      default: rtn_launch<8>(W, R, C, g, G, grid, scales, zeros, qweight, s); break;
     }
-#undef GPTQ_RTN_LAUNCH
     GPTQ_LAUNCH_CHECK();
     return GPTQ_OK;
   }

@@ -1153,3 +1153,73 @@ def test_rtn_of_wide_groups(B, bits, R, C, group):
     grids = [O.find_params(W16[:, j:j + g].astype(np.float64), bits, False) for j in range(0, C, g)]
     assert np.array_equal(out["scales"].cpu().numpy().astype(np.float64), np.stack([a for a, _ in grids], 1))
     assert np.array_equal(out["zeros"].cpu().numpy().astype(np.float64), np.stack([b for _, b in grids], 1))
+
+
+# Widest group of every form that keeps a group in registers (one warp with 4, 6 or 8 pieces a lane, 64 to 1024 threads with 8), and the next.
+RTN_EDGES = [1024, 1056, 1536, 1568, 2016, 2048, 4096, 4128, 6144, 6176, 8192, 8224, 12288, 12320, 16384, 24576, 24608, 32768, 32800, 49152, 49184]
+
+
+def _rtn_equals_oracle(W16, bits, group, out, sym=False):
+    codes, _ = O.rtn(W16, bits, group, sym)
+    assert np.array_equal(O.pack_codes(codes, bits), out["qweight"].cpu().numpy().view(np.uint32))
+    g = group if group > 0 else W16.shape[1]
+    grids = [O.find_params(W16[:, j:j + g].astype(np.float64), bits, sym) for j in range(0, W16.shape[1], g)]
+    assert np.array_equal(out["scales"].cpu().numpy().astype(np.float64), np.stack([a for a, _ in grids], 1))
+    assert np.array_equal(out["zeros"].cpu().numpy().astype(np.float64), np.stack([b for _, b in grids], 1))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 8])
+@pytest.mark.parametrize("C", RTN_EDGES)
+def test_rtn_at_the_widest_group_of_every_form(B, bits, C):
+    """Per-row grids of three rows, repeated beyond the 1024 groups at which narrower CTAs take over, and rows of two groups, bit for bit."""
+    W16 = (0.02 * np.random.default_rng(C + bits).standard_normal((3, C))).astype(np.float16)
+    _rtn_equals_oracle(W16, bits, 0, B.gptq_rtn_layer(torch.from_numpy(W16).cuda(), bits, 0, False))
+    out = B.gptq_rtn_layer(torch.from_numpy(W16).cuda().repeat(343, 1), bits, 0, False)
+    _rtn_equals_oracle(W16, bits, 0, {k: v[:3] for k, v in out.items()})
+    for v in out.values():
+        assert bool((v.view(-1, 3, v.shape[1]) == v[:3]).all())
+    W16 = (0.02 * np.random.default_rng(C).standard_normal((9, 2 * C))).astype(np.float16)
+    _rtn_equals_oracle(W16, bits, C, B.gptq_rtn_layer(torch.from_numpy(W16).cuda(), bits, C, False))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 8])
+@pytest.mark.parametrize("C,group", [(2048, 0), (2080, 0), (4096, 0), (5120, 0), (9216, 3072), (12288, 0), (40960, 0)])
+def test_rtn_of_a_large_matrix(B, bits, C, group):
+    """Beyond 1e8 weights a group that leaves many of its form's threads idle is read twice by one warp instead: seven rows, repeated."""
+    rows = (0.02 * np.random.default_rng(C + bits).standard_normal((7, C))).astype(np.float16)
+    W = torch.from_numpy(rows).cuda().repeat((2 ** 27 // C) // 7 + 2, 1)
+    assert W.numel() > 2 ** 27
+    out = B.gptq_rtn_layer(W, bits, group, False)
+    _rtn_equals_oracle(rows, bits, group, {k: v[:7] for k, v in out.items()})
+    for v in out.values():
+        assert bool((v.view(-1, 7, v.shape[1]) == v[:7]).all())
+
+
+@pytest.mark.parametrize("bits,sym,scale_fp16", [(2, False, False), (3, True, False), (4, False, True), (8, False, False), (O.BITS_TERNARY, True, False)])
+@pytest.mark.parametrize("C,group", [(2080, 0), (5120, 0), (8192, 4096), (8224, 0), (16416, 0), (49184, 0), (65568, 0)])
+def test_rtn_of_nan_and_infinity_in_different_warps(B, bits, C, group, sym, scale_fp16):
+    """A group on several warps: NaNs in the first warp's weights only, in a later one's only, in every weight; an infinity in another warp than a
+    NaN, of either sign.  The same rules as within a warp: a NaN has code 0 and no say in the grid, an infinity makes the scale infinite."""
+    rng = np.random.default_rng(C)
+    W = (0.02 * rng.standard_normal((8, C))).astype(np.float16)
+    g = group if group > 0 else C
+    bad = np.zeros(W.shape, dtype=bool)
+    bad[0, 5], bad[1, g - 3], bad[2, :g], bad[3, 300:304], bad[4, 2], bad[5, g - 1], bad[6, :300] = (True,) * 7
+    plain = np.where(bad, np.float16(0), W)                  # (0 lies inside every grid: the grid is that of the numbers)
+    codes_ref, _ = O.rtn(plain, bits, group, sym, scale_fp16=scale_fp16)
+    W = np.where(bad, np.float16(np.nan), W)
+    inf = np.zeros((8, C // g), dtype=bool)
+    for r, c, v in ((4, g - 2, np.inf), (5, 7, -np.inf), (6, 301, np.inf), (7, C - 9, -np.inf)):
+        W[r, c] = v
+        inf[r, c // g] = True
+    out = B.gptq_rtn_layer(torch.from_numpy(W).cuda(), bits, group, sym, scale_fp16=scale_fp16)
+    clean = B.gptq_rtn_layer(torch.from_numpy(plain).cuda(), bits, group, sym, scale_fp16=scale_fp16)
+    codes = O.unpack_codes(out["qweight"].cpu().numpy().view(np.uint32), bits, C)
+    scales, zeros = out["scales"].cpu().numpy(), out["zeros"].cpu().numpy()
+    of_inf = inf.repeat(g, 1)
+    assert np.array_equal(codes[~of_inf], np.where(bad, 0, codes_ref)[~of_inf])
+    for k, v in (("scales", scales), ("zeros", zeros)):
+        assert np.array_equal(v[~inf], clean[k].cpu().numpy()[~inf])
+    assert np.isposinf(scales[inf]).all()
+    z = np.nan_to_num(zeros).repeat(g, 1)                     # a number's quotient is 0 on such a scale
+    assert np.array_equal(codes[of_inf], np.where(np.isfinite(W), z, 0)[of_inf].astype(codes.dtype))
