@@ -87,8 +87,8 @@ struct TileItems {
   }
 };
 
-// Epilogues that add to what is there (kAccumulates; those that leave through TMA reductions all do): a tile's K may be cut as fine
-// as it pays.  The others get the whole K in one item.
+// Epilogues that add to what is there cheaply (kAccumulates; those that leave through TMA reductions all do): a tile's K may be cut as fine
+// as it pays.  The others get items of kSuperK, the whole of K in one if it is no longer than that.
 template <class T, class = void> struct accumulates { static constexpr bool value = pipe2::is_tile_epilogue<T>::value; };
 template <class T> struct accumulates<T, decltype((void)T::kAccumulates)> { static constexpr bool value = true; };
 

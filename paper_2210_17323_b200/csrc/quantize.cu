@@ -520,9 +520,10 @@ __global__ void residual_pair_kernel(const __half* __restrict__ W, const uint8_t
 
 // ---- contraction epilogue (one thread: one row, 32 consecutive columns of a partial sum) --------
 // Wblk[row][nofs + col ..) -= partial / (sE[row] sC[column]), as fp64 reductions: partial sums of one tile
-// come from several CTA pairs (one per super-chunk of the contraction).
+// come from several CTA pairs (one per super-chunk of the contraction).  Each costs 28 us per 256 x 256 tile (L2's fp64 rate), so K is not
+// cut below a super-chunk here, and up to 4096 earlier columns each element takes one sum, so that a call repeats itself bit for bit.
+// Per-inner-block form, 4-bit, K cut down to 512 / whole: 4096 x 4096 3.30 / 3.21 ms, 2048 x 8192 7.46 / 7.29; few rows 256 x 4096 2.81 / 2.87.
 struct EpiSubWblk {
-  static constexpr bool kAccumulates = true;
   double* Wblk; int64_t ldw; int nofs; int R, N;
   const float* sEinv; const float* sCinv;     // sCinv already offset to the first column of this contraction
   int stripe_major;                           // layout of Wblk (see wblk_from_w16_kernel)
