@@ -128,6 +128,8 @@ gptq_status_t gptq_hessian_symmetrize(float* H, int C, void* stream);
  *            the factor; [1] = which wait (61, 62: the panel launch; others: the contractions).
  * Computed as the inverse of the upper factor of H~ = U~ U~^T, which equals
  * Cholesky(H~^-1)^T by uniqueness of the Cholesky factor.
+ * For C <= 5120 every sum is formed in a fixed order: the same H gives the same U, bit for bit.  Beyond, sums over more than
+ * 4096 columns meet in memory in the order in which they are ready, and U may differ in its last bits from call to call.
  * Streams: for C > 1024 part of the work is enqueued on an internal stream (created once
  * per device on the first such call, never destroyed, it holds no device memory) that forks from
  * `stream` after the call's first kernels and joins it again before the call returns, so the
@@ -211,7 +213,9 @@ gptq_status_t gptq_prepare_hinv_static(const float* H, float damp, int C, float*
  *              The quantized weight is scales * (code - zeros).
  *   loss       double[1]: sum over all weights of E^2 = (w - q)^2 / U_jj^2 (Eq. 2 summed).
  *   dev_info   int[2], [0] = GPTQ_OK / GPTQ_ERR_NONFINITE / GPTQ_ERR_TIMEOUT.
- * All outputs are fully overwritten. */
+ * All outputs are fully overwritten.  The same W and U give the same codes, scales and zero-points for C <= 9216 (5120 in the
+ * per-inner-block form, see gptq_set_stage3_variant, and with groups of more than 2048 columns); beyond, update sums over more columns
+ * than that may meet in any order, as in gptq_prepare_hinv.  The loss is added up over rows in no fixed order. */
 size_t gptq_quantize_workspace_bytes(int R, int C, int bits, int group_size, int block);
 gptq_status_t gptq_quantize_layer(const void* W_fp16, const float* U, int R, int C,
                                   int bits, int group_size, int sym, int block,

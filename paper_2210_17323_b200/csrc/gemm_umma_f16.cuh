@@ -87,10 +87,27 @@ struct TileItems {
   }
 };
 
-// Epilogues that add to what is there cheaply (kAccumulates; those that leave through TMA reductions all do): a tile's K may be cut as fine
-// as it pays.  The others get items of kSuperK, the whole of K in one if it is no longer than that.
-template <class T, class = void> struct accumulates { static constexpr bool value = pipe2::is_tile_epilogue<T>::value; };
-template <class T> struct accumulates<T, decltype((void)T::kAccumulates)> { static constexpr bool value = true; };
+// Epilogues that may be called for several K ranges of one tile say so (kManyItems); the others need K in one item.
+template <class T, class = void> struct many_items { static constexpr bool value = false; };
+template <class T> struct many_items<T, decltype((void)T::kManyItems)> { static constexpr bool value = true; };
+
+// ---- cutting K -------------------------------------------------------------------------------------
+// A contraction of few tiles (a 1024-column block of a narrow layer, a diagonal block of the factor) leaves most CTA pairs without work
+// unless K is cut.  Its ranges then go to buffers of their own (EpiTileParts) and are added by a kernel after it, in the ranges' order: fp32 sums that several CTA pairs add to one element in memory come in no fixed order, so that two calls on the same input would
+// differ in the last bits, and every addition rounds at the size of what is there.  As many equal ranges as there are pairs for them
+// (so that no pair gets two), but none below 512, where an item's sums take as long to leave as to make (5 us a tile).
+struct Parts { int n; int k_item; };                  // n ranges of k_item (the last may be shorter); n = 0: more than kSuperK each
+constexpr int kPartPairs = 74;                         // CTA pairs of a B200
+inline int max_parts(int tiles, int64_t K) {
+  const int64_t by_k = (K + 255) / 512, by_pairs = kPartPairs / (tiles < kPartPairs ? tiles : kPartPairs);
+  const int64_t n = by_k < by_pairs ? by_k : by_pairs;
+  return n > 1 ? (int)n : 1;
+}
+inline Parts cut_k(int64_t K, int n) {
+  const int64_t kb = (K + BK - 1) / BK, per = (kb + n - 1) / n;
+  if (per > kSuperK / BK) return Parts{0, kSuperK};
+  return Parts{(int)((kb + per - 1) / per), (int)per * BK};
+}
 
 // Host-side description of one operand pair (hi, lo share the geometry).
 struct Operand {
@@ -98,14 +115,15 @@ struct Operand {
   int64_t rows, cols, ld;       // row-major [rows][cols], leading dimension ld (elements, a multiple of 8); cols = K
 };
 
-// acc = A * B^T over K = A.cols = B.cols; epi must accumulate (it is called once per super-chunk).
+// acc = A * B^T over K = A.cols = B.cols in items of k_item (a multiple of BK); epi is called once per item and must allow for several where
+// K is longer.
 template <bool kTriLeft, bool kUpperOut, class EpiF>
 gptq_status_t launch(const Operand& A, const Operand& B, int M, int N, EpiF epi, int* dev_info, cudaStream_t stream,
-                     int reserve_sms = 0, const CUtensorMap* out_map = nullptr) {
+                     int reserve_sms = 0, const CUtensorMap* out_map = nullptr, int k_item = kSuperK) {
   const int64_t K = A.cols;
   if (M <= 0 || N <= 0 || K <= 0) return GPTQ_OK;
-  static_assert(!pipe2::is_tile_epilogue<EpiF>::value || !kUpperOut, "tile epilogues write whole 32 x 32 blocks");
   if (pipe2::is_tile_epilogue<EpiF>::value != (out_map != nullptr)) return GPTQ_ERR_INVALID_ARG;
+  if (!many_items<EpiF>::value && K > k_item) return GPTQ_ERR_INVALID_ARG;
   Traits::Maps maps;
   if (out_map) maps.out = *out_map; else memset(&maps.out, 0, sizeof(maps.out));
   gptq_status_t st;
@@ -117,33 +135,20 @@ gptq_status_t launch(const Operand& A, const Operand& B, int M, int N, EpiF epi,
   if ((st = mk(&maps.a_lo, A.lo, A)) != GPTQ_OK) return st;
   if ((st = mk(&maps.b_hi, B.hi, B)) != GPTQ_OK) return st;
   if ((st = mk(&maps.b_lo, B.lo, B)) != GPTQ_OK) return st;
-  TileItems<kTriLeft, kUpperOut> items{(M + BM - 1) / BM, (N + BN - 1) / BN, (int)((K + BK - 1) / BK), kSuperK / BK};
-  if (accumulates<EpiF>::value) {
-    // Few tiles (a 1024-column block of a narrow layer, a diagonal block of the factor): K is cut until every CTA pair has an item, but
-    // not below 512, where an item's sums take as long to leave as to make.
-    const int tiles = kUpperOut ? items.tiles_m * (items.tiles_m + 1) / 2 : items.tiles_m * items.tiles_n, pairs = (device_sm_count() - reserve_sms) / 2;
-    while (items.sc_kb > 8 && tiles * ((items.kb_total + items.sc_kb - 1) / items.sc_kb) < pairs) items.sc_kb /= 2;
-  }
+  const TileItems<kTriLeft, kUpperOut> items{(M + BM - 1) / BM, (N + BN - 1) / BN, (int)((K + BK - 1) / BK), k_item / BK};
   const int n_sc = (items.kb_total + items.sc_kb - 1) / items.sc_kb;
   return pipe2::launch_pipe2<Traits>(maps, (int64_t)items.tiles_m * items.tiles_n * n_sc, items, epi, dev_info, stream,
                                      reserve_sms);
 }
 
-// Epilogue that leaves through TMA reductions: out[row][col] += alpha * sa[row] * sb[col] * partial (sa, sb optional) for
-// a row-major fp32 output described by Maps::out ({N, M}, 32 x 32 boxes, 128-byte swizzle).  The lanes write their rows
-// into the warp's swizzled 4 KB staging tile and one lane sends it off; elements beyond M or N are dropped by the TMA
-// unit.  L2 then adds whole 128-byte rows instead of 32 separate 16-byte pieces per instruction, which is what made
-// per-lane reductions cost 13 us per 256 x 256 tile (this form: 5 us).
-struct EpiTileAddF32 {
-  static constexpr bool kTile = true;
-  int M, N; float alpha;
+// Scaled sums of one warp's 32 x 32 block, sums * (alpha * sa[row]) * sb[col] (sa, sb optional), into its swizzled 4 KB staging tile.
+struct TileScale {
+  int M; float alpha;
   const float* sa; const float* sb;
-  __device__ __forceinline__ void tile(const Traits::Maps& maps, uint8_t* buf, int row0, int col0, const float (&v)[32],
-                                       int lane) const {
-    if (row0 >= M || col0 >= N) return;          // (warp-uniform)
+  __device__ __forceinline__ void stage(uint8_t* buf, int N, int row0, int col0, const float (&v)[32], int lane) const {
     const int row = row0 + lane;
     const float a = (sa != nullptr && row < M) ? alpha * sa[row] : alpha;
-    if (lane == 0) umma::bulk_group_wait_read_all();     // the previous reduction has read the staging tile
+    if (lane == 0) umma::bulk_group_wait_read_all();     // what was sent before has been read from the staging tile
     __syncwarp();
     const uint32_t base = umma::smem_u32(buf) + (uint32_t)lane * 128u;
 #pragma unroll
@@ -156,14 +161,41 @@ struct EpiTileAddF32 {
     }
     umma::fence_proxy_async();
     __syncwarp();
+  }
+};
+// Epilogue that leaves through TMA reductions: out[row][col] += scaled partial for a row-major fp32 output described by Maps::out ({N, M},
+// 32 x 32 boxes, 128-byte swizzle); elements beyond M or N are dropped by the TMA unit.  L2 then adds whole 128-byte rows instead of 32
+// separate 16-byte pieces per instruction, which is what made per-lane reductions cost 13 us per 256 x 256 tile (this form: 5 us).
+struct EpiTileAddF32 {
+  static constexpr bool kTile = true;
+  static constexpr bool kManyItems = true;
+  int N; TileScale scale;
+  __device__ __forceinline__ void tile(const Traits::Maps& maps, uint8_t* buf, int row0, int col0, const float (&v)[32], int lane, int /*kb0*/) const {
+    if (row0 >= scale.M || col0 >= N) return;            // (warp-uniform)
+    scale.stage(buf, N, row0, col0, v, lane);
     if (lane == 0) {
       umma::tma_reduce_add_2d(&maps.out, col0, row0, buf);
       umma::bulk_group_commit();
     }
   }
 };
+// Epilogue that stores the scaled sums of K range p = kb0 / sc_kb to part p of the output: Maps::out is {N, parts * rows}, `rows` the rows of
+// a part, a multiple of 32 (blocks are stored whole: what lies beyond M in a part is not read by anybody).
+struct EpiTileParts {
+  static constexpr bool kTile = true;
+  static constexpr bool kManyItems = true;
+  int N; TileScale scale; int rows, sc_kb;
+  __device__ __forceinline__ void tile(const Traits::Maps& maps, uint8_t* buf, int row0, int col0, const float (&v)[32], int lane, int kb0) const {
+    if (row0 >= scale.M || col0 >= N) return;            // (warp-uniform)
+    scale.stage(buf, N, row0, col0, v, lane);
+    if (lane == 0) {
+      umma::tma_store_2d(&maps.out, col0, (kb0 / sc_kb) * rows + row0, buf);
+      umma::bulk_group_commit();
+    }
+  }
+};
 // The tensor map such an epilogue needs: `out` points at the output's first element, ld in elements (a multiple of 4).
-inline gptq_status_t make_out_map_f32(CUtensorMap* m, float* out, int M, int N, int64_t ld) {
+inline gptq_status_t make_out_map_f32(CUtensorMap* m, float* out, int64_t M, int N, int64_t ld) {
   return make_tmap_2d(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, out, (uint64_t)N, (uint64_t)M, (uint64_t)ld * 4, 32, 32);
 }
 

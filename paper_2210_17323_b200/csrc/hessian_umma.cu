@@ -172,7 +172,7 @@ struct EpiAddTwiceTile {
   static constexpr bool kTile = true;
   int C;
   __device__ __forceinline__ void tile(const HessPairTraits::Maps& maps, uint8_t* buf, int row0, int col0,
-                                       const float (&v)[32], int lane) const {
+                                       const float (&v)[32], int lane, int /*kb0*/) const {
     if (row0 >= C || col0 >= C || col0 + 31 < row0) return;          // (warp-uniform)
     if (lane == 0) umma::bulk_group_wait_read_all();                  // the previous reduction has read the staging tile
     __syncwarp();

@@ -106,29 +106,6 @@ __global__ void inverse_row_scales_kernel(const float* __restrict__ U, int C, co
 
 // ---- tensor-core epilogues: one thread, one row, 32 consecutive columns of a partial sum ---------------
 // Every epilogue multiplies the partial sum by sa[row] * sb[col] (powers of two: the operands' scalings undone).
-// dst[row][cofs + col] -= partial for elements on or above the diagonal (fp32 reductions).
-struct EpiSubUpperRed {
-  static constexpr bool kAccumulates = true;
-  float* p; int64_t ld; int cofs; int M, N;
-  const float* sa; const float* sb;
-  __device__ __forceinline__ void operator()(int row, int col0, const float (&v)[32]) const {
-    if (row >= M || col0 >= N) return;
-    float* d = p + (int64_t)row * ld + cofs + col0;
-    const float a = -sa[row];
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-      const int c = cofs + col0 + 4 * g;            // global column of the group's first element
-      const float4 b = *reinterpret_cast<const float4*>(sb + col0 + 4 * g);
-      const float x0 = v[4 * g] * a * b.x, x1 = v[4 * g + 1] * a * b.y, x2 = v[4 * g + 2] * a * b.z, x3 = v[4 * g + 3] * a * b.w;
-      if (c >= row) umma::red_add_v4(d + 4 * g, x0, x1, x2, x3);
-      else if (c + 3 >= row) {
-        if (c + 1 >= row) atomicAdd(d + 4 * g + 1, x1);
-        if (c + 2 >= row) atomicAdd(d + 4 * g + 2, x2);
-        atomicAdd(d + 4 * g + 3, x3);
-      }
-    }
-  }
-};
 // dst[row][col] = partial * sa[row] * sb[col] * factor (fp32).  Only valid when the contraction is a single super-chunk.
 struct EpiStoreScaledF32 {
   float* p; int64_t ld; int M, N;
@@ -205,6 +182,24 @@ struct EpiStoreF32AndSplit {
   }
 };
 
+// D[r][c] -= sum over the n parts, in their order and in 64 bits, for c >= r (c, r < w <= 1024, w a multiple of 4).  One CTA per row.
+__global__ void __launch_bounds__(256) subtract_parts_kernel(float* __restrict__ D, int64_t ld, int w, const float* __restrict__ parts, int n,
+                                                             int64_t stride, int64_t ld_parts) {
+  const int r = blockIdx.x, c = 4 * threadIdx.x;
+  if (c >= w || c + 3 < r) return;
+  float4* d = reinterpret_cast<float4*>(D + (int64_t)r * ld + c);
+  const float4 old = *d;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int p = 0; p < n; ++p) {
+    const float4 v = *reinterpret_cast<const float4*>(parts + p * stride + r * ld_parts + c);
+    s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
+  }
+  float4 x;
+  x.x = c >= r ? (float)((double)old.x - s[0]) : old.x; x.y = c + 1 >= r ? (float)((double)old.y - s[1]) : old.y;
+  x.z = c + 2 >= r ? (float)((double)old.z - s[2]) : old.z; x.w = (float)((double)old.w - s[3]);
+  *d = x;
+}
 // dst{hi,lo}[r][c] = split(src[r][c] * sr[r] * sc[c]) for r < rows, c < w (w a multiple of 4; 16-byte aligned rows).
 __global__ void split_scaled_kernel(const float* __restrict__ src, int64_t ld_src, int rows, int w,
                                     const float* __restrict__ sr, const float* __restrict__ sc,
@@ -243,10 +238,17 @@ __global__ void split_diag_t_kernel(const float* __restrict__ U, int C, int j0, 
 }
 
 constexpr int kNB2 = 1024;   // outer panel width: contractions over everything outside it run on the tensor cores
+// K ranges of the update of a diagonal block by K later columns: 4 x 4 tiles (the six below the diagonal hold no work), cut as far as there are
+// CTA pairs, at least one range per super-chunk.  (Factor of 3072 / 4096 / 8192 columns: 1034 / 1443 / 3517 us with ranges of 4096 added in memory per
+// lane; 1021 / 1410 / 3414 with this and the pass that adds the ranges.)
+inline int schur_parts(int64_t K) {
+  const int n = f16x3::max_parts((kNB2 / f16x3::BM) * (kNB2 / f16x3::BN), K), least = ceil_div(K, f16x3::kSuperK);
+  return n > least ? n : least;
+}
 
 struct HinvWs {
   double* lam; panel::Flags* flags; double* pairs; __half* Fhi; __half* Flo; __half* VThi; __half* VTlo; __half* TThi; __half* TTlo;
-  __half* Vhi[2]; __half* Vlo[2]; __half* TAhi; __half* TAlo;
+  __half* Vhi[2]; __half* Vlo[2]; __half* TAhi; __half* TAlo; float* parts;
   float* r; float* rinv; float* rs; float* rsinv; float* u; float* uinv;      // [C] each
   float* g[2]; float* ginv[2]; float* gam; float* gam2inv;                     // [kNB2] each
   size_t bytes;
@@ -270,6 +272,7 @@ HinvWs carve_hinv(void* ws, int C) {
   }
   o.TAhi = w.take<__half>(outer ? (size_t)kNB2 * kNB2 : 0);       // split copy of the row block above a diagonal block
   o.TAlo = w.take<__half>(outer ? (size_t)kNB2 * kNB2 : 0);
+  o.parts = w.take<float>(outer ? (size_t)schur_parts(C - kNB2) * kNB2 * kNB2 : 0);   // sums of the K ranges of a diagonal block's update
   const size_t nc = outer ? (size_t)C : 0, np = outer ? (size_t)kNB2 : 0;
   o.r = w.take<float>(nc); o.rinv = w.take<float>(nc); o.rs = w.take<float>(nc); o.rsinv = w.take<float>(nc);
   o.u = w.take<float>(nc); o.uinv = w.take<float>(nc);
@@ -403,15 +406,21 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
       if (J + 2 < n_outer) GPTQ_CUDA_TRY(cudaStreamWaitEvent(s, as->b2[J + 2], 0));
       // C1
       f16x3::Operand A{w.Fhi + (int64_t)j0 * C + rows_p, w.Flo + (int64_t)j0 * C + rows_p, wj, K, C};
-      st = f16x3::launch<false, true>(A, A, wj, wj, EpiSubUpperRed{D, C, 0, wj, wj, w.rsinv + j0, w.rsinv + j0}, dev_info, s);
+      const f16x3::Parts cut = f16x3::cut_k(K, schur_parts(K));
+      CUtensorMap parts;
+      if ((st = f16x3::make_out_map_f32(&parts, w.parts, (int64_t)cut.n * kNB2, kNB2, kNB2)) != GPTQ_OK) return st;
+      st = f16x3::launch<false, true>(A, A, wj, wj, f16x3::EpiTileParts{wj, {wj, 1.f, w.rsinv + j0, w.rsinv + j0}, kNB2, cut.k_item / f16x3::BK},
+                                      dev_info, s, 0, &parts, cut.k_item);
       if (st != GPTQ_OK) return st;
+      subtract_parts_kernel<<<wj, 256, 0, s>>>(D, C, wj, w.parts, cut.n, (int64_t)kNB2 * kNB2, kNB2);
+      GPTQ_LAUNCH_CHECK();
       if (j0 > 0) {
         // B1
         GPTQ_CUDA_TRY(cudaStreamWaitEvent(sb, as->c4[J + 1], 0));
         f16x3::Operand A1{w.Fhi + rows_p, w.Flo + rows_p, j0, K, C};
         CUtensorMap out;
         if ((st = f16x3::make_out_map_f32(&out, U + j0, j0, wj, C)) != GPTQ_OK) return st;
-        st = f16x3::launch<false, false>(A1, A, j0, wj, f16x3::EpiTileAddF32{j0, wj, -1.f, w.rsinv, w.rsinv + j0}, dev_info, sb,
+        st = f16x3::launch<false, false>(A1, A, j0, wj, f16x3::EpiTileAddF32{wj, {j0, -1.f, w.rsinv, w.rsinv + j0}}, dev_info, sb,
                                          reserve, &out);
         if (st != GPTQ_OK) return st;
         GPTQ_CUDA_TRY(cudaEventRecord(as->b1[J], sb));
@@ -511,10 +520,12 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
     {
       f16x3::Operand A{w.Fhi, w.Flo, j0, j0, C};
       f16x3::Operand B{w.TThi, w.TTlo, wj, j0, C};
-      // partial = u_i gam_j' 2^-5 (sum_k U[i][k] T[j'][k])
+      // partial = u_i gam_j' 2^-5 (sum_k U[i][k] T[j'][k]).  Two halves of K where that gives every CTA pair at most one item: two sums
+      // onto zeros are the same in either order.
+      const int k_item = f16x3::max_parts(ceil_div(j0, f16x3::BM) * ceil_div(wj, f16x3::BN), j0) > 1 ? f16x3::cut_k(j0, 2).k_item : f16x3::kSuperK;
       CUtensorMap out;
       if ((st = f16x3::make_out_map_f32(&out, U + j0, j0, wj, C)) != GPTQ_OK) return st;
-      st = f16x3::launch<true, false>(A, B, j0, wj, f16x3::EpiTileAddF32{j0, wj, -1.f, w.uinv, w.gam2inv}, dev_info, s, 0, &out);
+      st = f16x3::launch<true, false>(A, B, j0, wj, f16x3::EpiTileAddF32{wj, {j0, -1.f, w.uinv, w.gam2inv}}, dev_info, s, 0, &out, k_item);
       if (st != GPTQ_OK) return st;
     }
     if (J + 1 < n_outer) {

@@ -115,6 +115,19 @@ __global__ void wblk_from_w16_kernel(const __half* __restrict__ W, int R, int C,
   const int64_t o = stripe_major ? ((int64_t)(r >> 7) * ldw + c) * 128 + (r & 127) : (int64_t)r * ldw + c;
   Wblk[o] = (double)__half2float(W[(int64_t)r * C + i2 + c]);
 }
+// D = the sum of n parts, `stride` floats apart, in their order and in 64 bits; the first part is D itself.  R rows of nb columns, four per thread.
+__global__ void __launch_bounds__(256) sum_parts_kernel(float* __restrict__ D, int R, int nb, int64_t ldd, int n, int64_t stride) {
+  const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (idx >= (int64_t)R * (nb / 4)) return;
+  float* d = D + idx / (nb / 4) * ldd + idx % (nb / 4) * 4;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+  for (int p = 0; p < n; ++p) {
+    const float4 v = *reinterpret_cast<const float4*>(d + p * stride);
+    s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
+  }
+  *reinterpret_cast<float4*>(d) = make_float4((float)s[0], (float)s[1], (float)s[2], (float)s[3]);
+}
 // The same for the stripe-major layout through a shared-memory tile of one stripe's 128 rows x 32 columns, so that both
 // the reads (along rows of W and D) and the writes (along a column of the stripe: 1 KB of consecutive doubles) are
 // coalesced and a thread has sixteen loads in flight; and with the lazy update folded in:
@@ -524,6 +537,7 @@ __global__ void residual_pair_kernel(const __half* __restrict__ W, const uint8_t
 // cut below a super-chunk here, and up to 4096 earlier columns each element takes one sum, so that a call repeats itself bit for bit.
 // Per-inner-block form, 4-bit, K cut down to 512 / whole: 4096 x 4096 3.30 / 3.21 ms, 2048 x 8192 7.46 / 7.29; few rows 256 x 4096 2.81 / 2.87.
 struct EpiSubWblk {
+  static constexpr bool kManyItems = true;
   double* Wblk; int64_t ldw; int nofs; int R, N;
   const float* sEinv; const float* sCinv;     // sCinv already offset to the first column of this contraction
   int stripe_major;                           // layout of Wblk (see wblk_from_w16_kernel)
@@ -574,6 +588,11 @@ inline int outer_block(int C, int group, int block) {
   return b2 < C ? b2 : C;
 }
 
+// Buffers for the fp32 sums of the lazy update of an outer block: one, or one for each of the K ranges that few rows are cut into.
+inline int lazy_tiles(int R, int B2) { return ceil_div(R, f16x3::BM) * ceil_div(B2, f16x3::BN); }
+inline int64_t lazy_rows(int R) { return (int64_t)ceil_div(R, 32) * 32; }
+inline size_t lazy_sum_floats(int R, int C, int B2) { return (size_t)f16x3::max_parts(lazy_tiles(R, B2), C) * (size_t)lazy_rows(R) * (size_t)B2; }
+
 }  // namespace
 }  // namespace gptq
 
@@ -593,7 +612,7 @@ extern "C" size_t gptq_quantize_workspace_bytes(int R, int C, int bits, int grou
   w.take<uint32_t>((size_t)C);                                    // column maxima of the scaled U
   w.take<float>((size_t)R);                                       // sE
   w.take<float>((size_t)R);                                       // 1 / sE
-  w.take<float>((size_t)R * outer_block(C, group_size, block));   // scaled fp32 sums of the lazy update of the outer block
+  w.take<float>(lazy_sum_floats(R, C, outer_block(C, group_size, block)));   // scaled fp32 sums of the lazy update of the outer block
   w.take<uint32_t>((size_t)C);                                    // factor form: column maxima above the diagonal blocks,
   w.take<float>((size_t)C);                                       //   sC2,
   w.take<float>((size_t)C);                                       //   1 / sC2
@@ -638,7 +657,7 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
   uint32_t* colmax = w.take<uint32_t>((size_t)C);
   float* sE = w.take<float>((size_t)R);
   float* sEinv = w.take<float>((size_t)R);
-  float* Dsum = w.take<float>((size_t)R * B2);
+  float* Dsum = w.take<float>(lazy_sum_floats(R, C, B2));
   uint32_t* colmax2 = w.take<uint32_t>((size_t)C);
   float* sC2 = w.take<float>((size_t)C);
   float* sC2inv = w.take<float>((size_t)C);
@@ -683,16 +702,29 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
     }
     // working weights of the outer block: original weights minus all updates from columns < i2
     if (stripe) {
-      // lazy update of the outer block: scaled fp32 sums from the tensor cores (added up in L2 by TMA reductions), then
-      // the fp64 working weights of the block in stripe-major order
+      // lazy update of the outer block: scaled fp32 sums from the tensor cores, then the fp64 working weights of the block in stripe-major
+      // order.  Few rows: K in ranges, each to a buffer of its own.  Many rows and more than a super-chunk of columns: the super-chunks'
+      // sums are added up in L2 by TMA reductions (two onto zeros in either order; more than 8192 columns in no fixed order).
       if (i2 > 0) {
-        GPTQ_CUDA_TRY(cudaMemsetAsync(Dsum, 0, (size_t)R * B2 * sizeof(float), s));
+        const int64_t rows = lazy_rows(R);
         f16x3::Operand A{Ehi, Elo, R, i2, C}, Bop{Phi, Plo, nb2, i2, C};
+        const f16x3::Parts cut = f16x3::cut_k(i2, f16x3::max_parts(lazy_tiles(R, B2), i2));
         CUtensorMap out;
-        gptq_status_t st = f16x3::make_out_map_f32(&out, Dsum, R, nb2, B2);
+        gptq_status_t st = f16x3::make_out_map_f32(&out, Dsum, cut.n > 0 ? cut.n * rows : R, nb2, B2);
         if (st != GPTQ_OK) return st;
-        st = f16x3::launch<false, false>(A, Bop, R, nb2, f16x3::EpiTileAddF32{R, nb2, 1.f, nullptr, nullptr}, dev_info, s, 0, &out);
+        const f16x3::TileScale plain{R, 1.f, nullptr, nullptr};
+        if (cut.n > 0) {
+          st = f16x3::launch<false, false>(A, Bop, R, nb2, f16x3::EpiTileParts{nb2, plain, (int)rows, cut.k_item / f16x3::BK}, dev_info, s, 0, &out,
+                                           cut.k_item);
+        } else {
+          GPTQ_CUDA_TRY(cudaMemsetAsync(Dsum, 0, (size_t)R * B2 * sizeof(float), s));
+          st = f16x3::launch<false, false>(A, Bop, R, nb2, f16x3::EpiTileAddF32{nb2, plain}, dev_info, s, 0, &out);
+        }
         if (st != GPTQ_OK) return st;
+        if (cut.n > 1) {
+          sum_parts_kernel<<<(unsigned)(((int64_t)R * (nb2 / 4) + 255) / 256), 256, 0, s>>>(Dsum, R, nb2, B2, cut.n, rows * B2);
+          GPTQ_LAUNCH_CHECK();
+        }
       }
       // (factor form: A holds the plain residuals and the panel rows above the block hold U~[before, blk] U_blk, scaled per
       // column by sC2: the sums ARE the block's correction, with the opposite sign)

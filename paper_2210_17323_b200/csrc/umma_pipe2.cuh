@@ -30,7 +30,7 @@ constexpr int threads_of(bool dynamic) { return dynamic ? 352 : 320; }
 constexpr int kThreads = threads_of(false);
 
 // Optional members: Traits::EPI_SMEM (bytes of shared memory for the epilogue, 1024-byte aligned, behind the stages) and
-// EpiF::kTile (the epilogue is called once per warp and 32 x 32 block of sums, with a 4 KB staging buffer of its own).
+// EpiF::kTile (the epilogue is called once per warp and 32 x 32 block of sums, with a 4 KB staging buffer of its own and the item's first K block).
 template <class T, class = void> struct epi_smem_of { static constexpr int value = 0; };
 template <class T> struct epi_smem_of<T, decltype((void)T::EPI_SMEM)> { static constexpr int value = T::EPI_SMEM; };
 template <class T, class = void> struct is_tile_epilogue { static constexpr bool value = false; };
@@ -285,7 +285,7 @@ umma_pipe2_kernel(const __grid_constant__ typename Traits::Maps maps, const int 
 #pragma unroll
         for (int c = 0; c < 4; ++c)
           epi.tile(maps, epi_smem + (warp - 2) * 4096, m0 + BM_CTA * (int)rank + q * 32, n0 + half * 128 + 32 * c,
-                   *reinterpret_cast<const float(*)[32]>(&sum[32 * c]), lane);
+                   *reinterpret_cast<const float(*)[32]>(&sum[32 * c]), lane, kb0);
       } else {
         const int row = m0 + BM_CTA * (int)rank + q * 32 + lane;
 #pragma unroll

@@ -1,4 +1,6 @@
 """GPU parity: the CUDA path (through the C ABI) against the fp64 oracle, element by element."""
+import functools
+
 import numpy as np
 import pytest
 
@@ -1223,3 +1225,77 @@ def test_rtn_of_nan_and_infinity_in_different_warps(B, bits, C, group, sym, scal
     assert np.isposinf(scales[inf]).all()
     z = np.nan_to_num(zeros).repeat(g, 1)                     # a number's quotient is 0 on such a scale
     assert np.array_equal(codes[of_inf], np.where(np.isfinite(W), z, 0)[of_inf].astype(codes.dtype))
+
+
+def _factor_inputs(C, tokens, seed=0):
+    """A Hessian of `tokens` activations with a spread of channel scales, summed by torch (the same bits for every call on it)."""
+    g = torch.Generator("cuda").manual_seed(seed + C)
+    X = torch.randn((tokens, C), device="cuda", generator=g) * torch.exp(torch.randn(C, device="cuda", generator=g))
+    H = 2.0 * X.T @ X
+    return (H + H.T) / 2
+
+
+@pytest.mark.parametrize("factor", [False, True])
+@pytest.mark.parametrize("C", [1568, 2048, 2304, 3072, 4096, 5120])
+def test_stage_2_repeats_itself_bit_for_bit(B, factor, C):
+    """Up to 4096 columns behind a diagonal block, contractions whose K is cut are added in a fixed order: the same H gives the same factor."""
+    H = _factor_inputs(C, 2 * C)
+    ref, info = B.gptq_prepare_hinv(H, 0.01, factor=factor)
+    for _ in range(5):
+        U, _ = B.gptq_prepare_hinv(H, 0.01, factor=factor)
+        assert torch.equal(U, ref)
+    assert info.tolist()[0] == 0
+
+
+@pytest.mark.parametrize("R,C,bits,group,block,factor", [(1000, 2400, 3, 32, 64, True), (768, 3072, 4, 0, 128, False), (33, 4128, 3, 96, 32, False),
+                                                         (2000, 8192, 2, 64, 128, True), (64, 12288, 4, 0, 128, True), (200, 3072, 3, 128, 128, None)])
+def test_stage_3_repeats_itself_bit_for_bit(B, R, C, bits, group, block, factor):
+    """The lazy update of few rows (K cut) and of up to 8192 earlier columns of many: the same codes, scales and zero-points, call after call.
+    factor None: the per-inner-block form."""
+    H = _factor_inputs(C, 2 * C)
+    W = torch.from_numpy(_layer(R, C, 64, cfg=16).w()).cuda()
+    F, _ = B.gptq_prepare_hinv(H, 0.01, factor=bool(factor))
+    quantize = functools.partial(B.gptq_quantize_layer, factor=bool(factor))
+    old = B.gptq_set_stage3_variant(0 if factor is None else 1)
+    try:
+        ref = quantize(W, F, bits, group, False, block)
+        for _ in range(5):
+            out = quantize(W, F, bits, group, False, block)
+            for k in ("qweight", "scales", "zeros"):
+                assert torch.equal(out[k], ref[k]), k
+    finally:
+        B.gptq_set_stage3_variant(old)
+
+
+@pytest.mark.parametrize("R", [1, 31, 33, 257, 1000])
+@pytest.mark.parametrize("C,factor", [(1568, False), (2400, True), (4128, False), (5632, True)])
+def test_few_rows_give_what_they_give_among_many(B, R, C, factor):
+    """Rows are independent: alone (K of the lazy update in ranges, row counts around the 32 of a range's buffer) and as the first rows of 5000
+    (K whole) they differ by the rounding of fp32 sums, which moves a code on a tie at most."""
+    H = _factor_inputs(C, 2 * C)
+    W = torch.from_numpy(_layer(5000, C, 64, cfg=16).w()).cuda()
+    F, _ = B.gptq_prepare_hinv(H, 0.01, factor=factor)
+    quantize = functools.partial(B.gptq_quantize_layer, factor=factor)
+    few, many = quantize(W[:R].contiguous(), F, 4, 0, False, 128), quantize(W, F, 4, 0, False, 128)
+    a = O.unpack_codes(few["qweight"].cpu().numpy().view(np.uint32), 4, C)
+    b = O.unpack_codes(many["qweight"][:R].cpu().numpy().view(np.uint32), 4, C)
+    assert torch.equal(few["scales"], many["scales"][:R])
+    assert (a == b).mean() >= 0.999 and np.abs(a.astype(int) - b).max() <= 1
+
+
+@pytest.mark.parametrize("C,tokens,damp", [(2304, 1152, 1e-3), (4096, 2048, 1e-3), (3072, 6144, 0.01)])
+def test_stage_2_against_64_bits(B, C, tokens, damp):
+    """Widths whose contractions are cut, Hessians of half as many tokens as channels among them.  What fp32 input alone does to U: the same factor of
+    the damped Hessian with every entry moved by up to half a unit in the last place, 2^-24 of it.  The fp16-pair contractions' sums are
+    good to 1e-6 (17 x 2^-24: three products of 22-bit operands, 128 of them at a time in a truncating accumulator), and an entry passes through
+    two, the Schur complement's and its panel's product: 34 times that.  (Measured: 15 to 18 times, single rows 17 to 20.)"""
+    H = _factor_inputs(C, tokens)
+    Hd = H.double() + damp * H.diagonal().double().mean() * torch.eye(C, device="cuda", dtype=torch.float64)
+    g = torch.Generator("cuda").manual_seed(1)
+    noise = torch.triu(torch.rand((C, C), device="cuda", generator=g, dtype=torch.float64) * 2 - 1) * 2.0 ** -24
+    ref, moved = (torch.linalg.cholesky(torch.linalg.inv(M)).T for M in (Hd, Hd * (1 + noise + torch.triu(noise, 1).T)))
+    U, info = B.gptq_prepare_hinv(H, damp)
+    assert info.tolist()[0] == 0
+    err, sens = ((x.double() - ref).norm() / ref.norm() for x in (U, moved))
+    rows, sens_rows = (((x.double() - ref).norm(dim=1) / ref.norm(dim=1)).max() for x in (U, moved))
+    assert float(err / sens) <= 34 and float(rows / sens_rows) <= 34
