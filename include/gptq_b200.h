@@ -213,9 +213,9 @@ gptq_status_t gptq_prepare_hinv_static(const float* H, float damp, int C, float*
  *              The quantized weight is scales * (code - zeros).
  *   loss       double[1]: sum over all weights of E^2 = (w - q)^2 / U_jj^2 (Eq. 2 summed).
  *   dev_info   int[2], [0] = GPTQ_OK / GPTQ_ERR_NONFINITE / GPTQ_ERR_TIMEOUT.
- * All outputs are fully overwritten.  The same W and U give the same codes, scales and zero-points for C <= 9216 (5120 in the
- * per-inner-block form, see gptq_set_stage3_variant, and with groups of more than 2048 columns); beyond, update sums over more columns
- * than that may meet in any order, as in gptq_prepare_hinv.  The loss is added up over rows in no fixed order. */
+ * All outputs are fully overwritten.  The same W and U give the same codes, scales and zero-points for C <= 8192 (4096 in the
+ * per-inner-block form, see gptq_set_stage3_variant, and with groups of more than 2048 columns); beyond, update sums over more
+ * columns may meet in any order, as in gptq_prepare_hinv.  The loss is added up over rows in no fixed order. */
 size_t gptq_quantize_workspace_bytes(int R, int C, int bits, int group_size, int block);
 gptq_status_t gptq_quantize_layer(const void* W_fp16, const float* U, int R, int C,
                                   int bits, int group_size, int sym, int block,

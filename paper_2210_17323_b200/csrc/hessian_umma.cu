@@ -8,10 +8,10 @@
 // is exactly the canonical MN-major 128B-swizzle layout (8-token groups 1024 B apart, 64-channel
 // groups one box = 8192 B apart).
 //
-// Work decomposition: output tiles of 128 x 256 that touch the upper triangle, times super-chunks
-// of up to 16384 tokens.  Accumulation is hierarchical: 512 tokens (32 MMAs) in a TMEM accumulator,
-// chunk sums added round-to-nearest in registers over the super-chunk, super-chunk sums added to H
-// with vector reductions (red.global.add.v4.f32).
+// Work decomposition: output tiles that touch the upper triangle, 256 x 256 on CTA pairs (128 x 256 on single CTAs below 512
+// channels), times token ranges of up to 8192 tokens (one-CTA path: 16384).  Accumulation is hierarchical: 512 tokens (32 MMAs)
+// in a TMEM accumulator, chunk sums added round-to-nearest in registers over the range, the ranges' sums added to H in memory
+// by TMA tile reductions (one-CTA path: vector reductions per lane).
 #include "hessian_umma.cuh"
 #include "umma_pipe.cuh"
 #include "umma_pipe2.cuh"

@@ -30,8 +30,8 @@
 // Threads: warps 0-3 own the rows (thread t <-> row t <-> TMEM lane t); warp 4 issues the near pushes, warp 5 the far ones,
 // warp 6 stages U's diagonal blocks, warp 7 has nothing to do, warps 8-11 drain the far pushes.  A row thread needs 200
 // registers and more (32 doubles of weights); at 168 the loads that run ahead are spilled, and so waited for.  So the three
-// warpgroups share out the registers anew: 248 + 112 + 136 of the 3 x 168 the kernel is launched with.  (The instance without
-// small groups still spills 20 bytes somewhere, the other one none.)
+// warpgroups share out the registers anew: 248 + 112 + 136 of the 3 x 168 the kernel is launched with.
+// Neither instance spills.
 #pragma once
 
 constexpr int kStripeRows = 128;
@@ -591,7 +591,8 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
         // w / scale + 1/2 is formed with the reciprocal, added to 2^32 + 2048: the low word then holds it in units of 2^-20,
         // its upper twelve bits the code (rounded, counted from zero-point - 2048), to be clamped as an integer.  With U's row
         // divided by U_jj (n) the next column's weight is (w' - w n) + (scale n) (code - zero-point): everything but the last
-        // multiply-add is ready when the code is.  The other columns take (w - scale (code - zero-point)) n, exact in its one
+        // multiply-add is ready when the code is.  (w n is formed before it cancels: the next weight's rounding error is 2^-53 of |w n|, not of
+        // |w - q| n: 2^-29 of the fp32-level sums that weight has met.)  The other columns take (w - scale (code - zero-point)) n, exact in its one
         // multiply-add (24-bit scale).  Where the quotient lies within 2^-20 of a tie (the fraction bits are next to zero) or
         // outside twelve bits (the upper word is another one), the sixteen columns are done again with the division itself.
         // (rint, fmin and fmax take 20 to 25 cycles each in fp64.)  The errors' way into the tile fills the chain's gaps, pair by
