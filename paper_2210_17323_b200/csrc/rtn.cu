@@ -181,6 +181,7 @@ __device__ __forceinline__ void rtn_store_words(uint32_t* qrow, int i, bool on, 
 // a CTA, or a CTA per group.  A group's load, minimum, grid and codes follow one another, so what counts is how many bytes of W an SM has
 // on their way: the pieces fill the threads (kHeld and kThreads follow the group's width, see rtn_launch) and the minimum of CTAs per SM keeps a
 // thread at 64 registers, 80 where a warp holds 6 or 8 (512 threads, 32768 columns: 2 CTAs an SM instead of 1, 107 instead of 154 us for 1.5e8 weights).
+// (Spilled: 16 bytes in the 2- and 3-bit instances of 1024 threads, 8 in those of 768; nothing elsewhere.)
 // 12288 x 12288, 4-bit: 90 us, where the bytes alone take 57 (192 threads; with 256 of them a quarter idle 103; rtn_fused_kernel, which reads W
 // twice, half of it from DRAM: 112; a ring in shared memory that asynchronous copies fill one row ahead: 121).
 template <int F, int kThreads, int kHeld>
