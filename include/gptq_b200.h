@@ -125,7 +125,7 @@ gptq_status_t gptq_hessian_symmetrize(float* H, int C, void* stream);
  *            tensor-core contractions use for C > 1024 (a Hessian so ill-conditioned that entries of
  *            the inverse factor exceed ~100 times their row's diagonal entry); [1] = a row index.
  *            GPTQ_ERR_TIMEOUT, at any C: a bounded wait inside one of the kernels ran out and U is not
- *            the factor; [1] = which wait (61, 62: the panel launch; others: the contractions).
+ *            the factor; [1] = which wait (61 to 63: the panel launch; others: the contractions).
  * Computed as the inverse of the upper factor of H~ = U~ U~^T, which equals
  * Cholesky(H~^-1)^T by uniqueness of the Cholesky factor.
  * For C <= 5120 every sum is formed in a fixed order: the same H gives the same U, bit for bit.  Beyond, sums over more than

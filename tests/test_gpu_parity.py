@@ -237,6 +237,29 @@ def test_panel_factorisation_at_tile_edges(B, C):
             assert ((U - ref).norm(dim=1) / ref.norm(dim=1)).max() <= 1e-4
 
 
+@pytest.mark.parametrize("C", [64, 128, 160])
+@pytest.mark.parametrize("exponent", [0, 20, 55])
+def test_panel_pivots_over_the_range(B, C, exponent):
+    """H scaled by powers of two between 2^-exponent and 2^exponent per row and column (pivots from 2^-110 to 2^110) has the scaled factor: U's
+    column j over s_j, every bit the same.  The last pivot that is not positive is reported: a zero or negative diagonal entry, or the last
+    column where one is no number or infinite (the dampening, 0 times their mean, is no number then)."""
+    r = np.random.default_rng(5 * C + exponent)
+    X = r.standard_normal((3 * C, C))
+    H = torch.from_numpy((2 * X.T @ X).astype(np.float32)).cuda()
+    s = torch.from_numpy(np.ldexp(1.0, r.integers(-exponent, exponent + 1, C)).astype(np.float32)).cuda()
+    U, info = B.gptq_prepare_hinv(H, 0.0)
+    V, info2 = B.gptq_prepare_hinv(H * s[:, None] * s[None, :], 0.0)
+    torch.cuda.synchronize()
+    assert info.tolist() == [0, 0] and info2.tolist() == [0, 0]
+    assert torch.equal(V * s[None, :], U)
+    for j, d, where in ((C - 1, 0.0, C - 1), (C - 9, -1.0, C - 9), (7, float("nan"), C - 1), (0, float("inf"), C - 1)):
+        bad = H.clone()
+        bad[j, j] = d
+        _, info = B.gptq_prepare_hinv(bad, 0.0)
+        torch.cuda.synchronize()
+        assert info.tolist() == [B.ERR_NOT_PD, where], (j, d, info.tolist())
+
+
 @pytest.mark.parametrize("C", [32, 64, 96, 128])
 @pytest.mark.parametrize("tokens_per_channel,damp", [(2.0, 0.01), (0.5, 1e-3)])
 def test_a_block_of_128_columns_is_factored_in_64_bits(B, C, tokens_per_channel, damp):
