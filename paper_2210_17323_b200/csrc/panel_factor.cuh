@@ -21,8 +21,8 @@
 // products of a step (about 1000 DMMAs of 16 cycles on three quarters of the SM) in warps that run beside it, each with a row of pieces
 // in registers; T T^T and the inverse, which nothing else waits for, follow at their own pace.
 // Measured, columns of one call: as separate launches 768 / 1024 0.94 / 1.29 ms; this list with a chain of eight warps that met at a barrier
-// twice every eight columns, roots on it, 0.189 / 0.247 (30,600 cycles a step); this form 0.145 / 0.190 (21,000, of which 17,500 the chain's
-// own and the rest waiting for products).  Products as halves of 32 rows, three flags looked at at once: 0.159 / 0.209 with whole ones.
+// twice every eight columns, roots on it, 0.189 / 0.247 (30,600 cycles a step); this form 0.141 / 0.182 (20,000, of which 17,500 the chain's
+// own and the rest waiting for products).
 #pragma once
 
 namespace gptq {
@@ -41,10 +41,12 @@ constexpr int kPairV1 = 0, kPairT = 1, kPairV0 = 2, kPairTiles = 3;
 
 // Progress of one launch, in the caller's workspace; all zero when the kernel starts.
 struct Flags {
+  int factored;                      // tile columns factored so far (from the last one); on a line of its own, which most of the waiting look at
+  int unused[31];
   int role;                          // order of arrival: 0 runs the chain
-  int ticket;                        // next entry of the list of products
-  int factored;                      // tile columns factored so far (from the last one)
+  int ticket;                        // next half of an entry of the list of products
   int abort;                         // a wait ran out: everybody leaves
+  int unused2[21];
   int solved[kMaxTiles * kMaxTiles]; // halves of tile (i, k) that have been through step k's solve
   int updated[kMaxTiles * kMaxTiles];// updates applied to halves of tile (i, c)
   int paired[kMaxTiles / 2];         // the fp64 tiles of pair (2 m, 2 m + 1) are complete
@@ -67,7 +69,10 @@ struct TaskSmem {
     struct { float As[32][LDF]; float Bs[TB][LDF]; };
     double E[TB][LDD];
   };
-  double P[TB][LDD];
+  union {
+    double P[TB][LDD];
+    float sums[2][2][4][128];
+  };
   int msg[4];
 };
 struct ChainSmem {
@@ -89,15 +94,21 @@ struct Smem {
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 // Named barriers.  Of a step of the chain: V_g of panel jb is there (1 + jb % 2), its Y is (3), the chain's next two pieces are (4), the
-// step's tiles have been read (5), the warps that fetch tiles (6), those that hand the last rows of V out (7), the roots of a panel (9).
+// step's tiles have been read (5), the warps that fetch tiles (6), those that hand the last rows of V out (7), the roots of a panel (9), the
+// next step's tiles are there (10).
 // Of products: 8.
-constexpr int kBarV = 1, kBarY = 3, kBarNext = 4, kBarRead = 5, kBarFetch = 6, kBarOut = 7, kBarGroup = 8, kBarRoot = 9;
+constexpr int kBarV = 1, kBarY = 3, kBarNext = 4, kBarRead = 5, kBarFetch = 6, kBarOut = 7, kBarGroup = 8, kBarRoot = 9, kBarTiles = 10;
 constexpr int kRows = 8 * 32, kFetch = 3 * 32, kOut = 3 * 32;   // threads that own a row of pieces; that fetch; that hand the last rows out
 
 // ---- waiting -------------------------------------------------------------------------------------
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ int ld_relaxed(const int* p) {
+  int v;
+  asm volatile("ld.relaxed.gpu.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_release(int* p, int v) {
@@ -111,6 +122,7 @@ __device__ __forceinline__ void add_release(int* p, int v) {
 __device__ __forceinline__ bool wait_all_ge(const int* p, int v, int n, const Args& a) {
   const int lane = threadIdx.x & 31;
   uint64_t t0 = 0;
+  uint32_t looks = 0;
   for (;;) {
     if (__all_sync(0xffffffffu, lane >= n || ld_acquire(p) >= v)) return true;
     const uint64_t now = umma::global_timer_ns();
@@ -123,10 +135,11 @@ __device__ __forceinline__ bool wait_all_ge(const int* p, int v, int n, const Ar
         st_release(&a.fl->abort, 1);
       }
       out = true;
-    } else if (lane == 0) {
+    } else if (lane == 0 && (++looks & 15) == 0) {
       out = ld_acquire(&a.fl->abort) != 0;
     }
     if (__any_sync(0xffffffffu, out)) return false;
+    __nanosleep(40);                                     // (a hundred warps wait like this one, and a look delays the others')
   }
 }
 
@@ -166,21 +179,23 @@ __host__ __device__ inline int tasks_before_step(int nt, int k) {
 __host__ __device__ __forceinline__ int updates_before(int nt, int i, int c, int k) { return i <= c ? nt - 1 - k : i - k; }
 
 // ---- tile products (fp32) ------------------------------------------------------------------------------
-// 32 rows of a tile product: acc[p][q] = sum_m As[ty + 16 p][m] * Bs[tx + 16 q][m]
-__device__ __forceinline__ void product(const float (*As)[LDF], const float (*Bs)[LDF], float (&acc)[2][4], int tx, int ty) {
+// 32 rows of a tile product by 256 threads, half of the 64 products of an entry by each 128 of them: acc[p][q] = sum_m As[ty + 8 p][m] *
+// Bs[tx + 16 q][m] over the half's m.  What bounds it is the shared-memory pipe, four cycles per 16-byte load and warp: 64 loads a thread
+// (with 2 x 4 entries a thread and all 64 products 96, 2700 cycles; 768 / 1024 columns 142 / 185 us against 141 / 182).
+__device__ __forceinline__ void product(const float (*As)[LDF], const float (*Bs)[LDF], float (&acc)[4][4], int tx, int ty, int m0) {
 #pragma unroll
-  for (int p = 0; p < 2; ++p)
+  for (int p = 0; p < 4; ++p)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[p][q] = 0.f;
 #pragma unroll
-  for (int m = 0; m < TB; m += 4) {
-    float4 x[2], y[4];
+  for (int m = 0; m < TB / 2; m += 4) {
+    float4 x[4], y[4];
 #pragma unroll
-    for (int p = 0; p < 2; ++p) x[p] = *reinterpret_cast<const float4*>(&As[ty + 16 * p][m]);
+    for (int p = 0; p < 4; ++p) x[p] = *reinterpret_cast<const float4*>(&As[ty + 8 * p][m0 + m]);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) y[q] = *reinterpret_cast<const float4*>(&Bs[tx + 16 * q][m]);
+    for (int q = 0; q < 4; ++q) y[q] = *reinterpret_cast<const float4*>(&Bs[tx + 16 * q][m0 + m]);
 #pragma unroll
-    for (int p = 0; p < 2; ++p)
+    for (int p = 0; p < 4; ++p)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         acc[p][q] = fmaf(x[p].x, y[q].x, acc[p][q]); acc[p][q] = fmaf(x[p].y, y[q].y, acc[p][q]);
@@ -289,7 +304,7 @@ __device__ __forceinline__ bool pair_inverse(const Args& a, TaskSmem& s, int k, 
 // One half (rows 32 half .. 32 half + 31) of an entry of the list, 256 threads.  False if the launch is being abandoned.  (A pair's inverse
 // is made whole, with the first half.)
 __device__ __forceinline__ bool run_task(const Args& a, TaskSmem& s, const Task& k, int half, int t) {
-  const int nt = a.nt, tx = t & 15, ty = t >> 4;
+  const int nt = a.nt, tx = t & 15, ty = (t >> 4) & 7, h = t >> 7;
   Flags* fl = a.fl;
   if (k.c + 1 == k.k && (k.k & 1) && k.i == k.k) return true;                     // part of pair_inverse
   if (k.kind == 0 && k.i == k.k + 1 && !(k.k & 1)) return half != 0 || pair_inverse(a, s, k.k, t);
@@ -304,29 +319,37 @@ __device__ __forceinline__ bool run_task(const Args& a, TaskSmem& s, const Task&
   }
   bar_sync(kBarGroup, kGroup);                          // (also: the previous product is done with As and Bs)
   if (!s.msg[3]) return false;
-  const int r0 = 32 * half;
-  float* out = a.A + (int64_t)(TB * k.i + r0 + ty) * a.ld + TB * k.c + tx;
+  const int r0 = 32 * half, row = r0 + ty + 16 * h;      // this thread's results: rows row and row + 8, columns tx + 16 q
+  float* out = a.A + (int64_t)(TB * k.i + row) * a.ld + TB * k.c + tx;
   float old[2][4];
 #pragma unroll
   for (int p = 0; p < 2; ++p)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       old[p][q] = 0.f;
-      if (k.kind == 1 && !own && TB * k.i + r0 + ty + 16 * p < a.w && TB * k.c + tx + 16 * q < a.w)
-        old[p][q] = __ldcg(out + (int64_t)(16 * p) * a.ld + 16 * q);
+      if (k.kind == 1 && !own && TB * k.i + row + 8 * p < a.w && TB * k.c + tx + 16 * q < a.w)
+        old[p][q] = __ldcg(out + (int64_t)(8 * p) * a.ld + 16 * q);
     }
   load_tile<TB>(a, k.kind == 0 ? k.k : k.c, k.k, 0, s.Bs, t);
   if (own) load_tile_t(a, k.k, k.k, r0, s.As, t); else load_tile<32>(a, k.i, k.k, r0, s.As, t);
   copy_async_wait();
   bar_sync(kBarGroup, kGroup);
-  float acc[2][4];
-  product(s.As, s.Bs, acc, tx, ty);
+  float acc[4][4];
+  product(s.As, s.Bs, acc, tx, ty, TB / 2 * h);
+  // the other half's rows (p = 0, 1 belong to h = 0, p = 2, 3 to h = 1) through shared memory
 #pragma unroll
   for (int p = 0; p < 2; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (TB * k.i + r0 + ty + 16 * p < a.w && TB * k.c + tx + 16 * q < a.w)
-        out[(int64_t)(16 * p) * a.ld + 16 * q] = k.kind == 0 ? acc[p][q] : old[p][q] - acc[p][q];
+    for (int q = 0; q < 4; ++q) s.sums[h][p][q][t & 127] = h ? acc[p][q] : acc[p + 2][q];
+  bar_sync(kBarGroup, kGroup);
+#pragma unroll
+  for (int p = 0; p < 2; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float v = (h ? acc[p + 2][q] : acc[p][q]) + s.sums[h ^ 1][p][q][t & 127];
+      if (TB * k.i + row + 8 * p < a.w && TB * k.c + tx + 16 * q < a.w)
+        out[(int64_t)(8 * p) * a.ld + 16 * q] = k.kind == 0 ? v : old[p][q] - v;
+    }
   bar_sync(kBarGroup, kGroup);
   if (t == 0)                                           // (the release covers what the barrier has collected from all threads)
     add_release(k.kind == 0 ? &fl->solved[k.i * kMaxTiles + k.k] : &fl->updated[k.i * kMaxTiles + k.c], 1);
@@ -704,7 +727,7 @@ __device__ __forceinline__ void chain_solve(const Args& a, ChainSmem& s, int k, 
   }
 }
 // Tiles (k, k) and, unless k is the last column, (k, k + 1) to s.Md and s.Mx by n threads (a multiple of 16): asynchronous copies, zeros
-// beyond the block, whose last rows of s.Md are those of the identity.
+// beyond the block, whose last rows of s.Md are those of the identity.  The caller waits for the copies.
 __device__ __forceinline__ void load_chain_tiles(const Args& a, ChainSmem& s, int k, int t, int n) {
   const int c = 4 * (t & 15), step = n >> 4;
   const bool next = k + 1 < a.nt, in0 = TB * k + c < a.w, in1 = next && TB * (k + 1) + c < a.w;
@@ -716,7 +739,6 @@ __device__ __forceinline__ void load_chain_tiles(const Args& a, ChainSmem& s, in
     if (in1) copy_async_16(&s.Mx[row][c], src + TB);
     else if (next) *reinterpret_cast<float4*>(&s.Mx[row][c]) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  copy_async_wait();
 }
 // Three warps beside the factorisation of tile k: they hand out T[k][k + 1] (in 64 bits to the pair's tile), then fetch the next step's
 // tiles, if they are ready before the chain is.  (t: 0 .. 95)
@@ -738,15 +760,17 @@ __device__ __forceinline__ void chain_fetch(const Args& a, ChainSmem& s, int k, 
   }
   bar_sync(kBarRead, 32 + kRows + kFetch);
   if (k == 0) return;
-  if (t == 0) {
+  if (warp == 0) {
     const int* p = &a.fl->updated[(k - 1) * kMaxTiles + k - 1];
     bool ready = false;
-    while (!(ready = ld_acquire(p) >= 2 * (nt - 1 - k) && ld_acquire(p + 1) >= 2 * (nt - 1 - k)))
-      if (*reinterpret_cast<volatile int*>(&s.done) == k) break;
-    if (ready) s.got = k - 1;
+    while (!(ready = __all_sync(0xffffffffu, lane > 1 || ld_relaxed(p + lane) >= 2 * (nt - 1 - k))))
+      if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&s.done) == k)) break;       // (then all threads fetch, see run_chain)
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    if (t == 0 && ready) s.got = k - 1;
   }
   bar_sync(kBarFetch, kFetch);
   if (s.got == k - 1) load_chain_tiles(a, s, k - 1, t, kFetch);
+  // (a bulk copy per row into an mbarrier instead of 16-byte copies: 1024 columns 195 us against 182)
 }
 
 // All threads.  Warps by role: T[k][k + 1] is made by warps 0 - 3 and 8 - 11, while 13 - 15 hand the last rows of the step before out; then
@@ -777,7 +801,10 @@ __device__ __forceinline__ bool run_chain(const Args& a, Smem& sm, int t) {
   for (int k = nt - 1; k >= 0; --k) {
     const bool first = k == nt - 1;
     if (!first) hand_out(k + 1);
-    if (s.got != k) {
+    if (s.got == k) {                                    // (the word goes out before the last tiles are in)
+      if ((warp & 3) == 0 && warp > 0) copy_async_wait();
+      if ((warp & 4) == 0 || (warp & 3) == 0) bar_sync(kBarTiles, 10 * 32);
+    } else {
       if (!first) {
         if (t < kGroup) {
           const bool go = chain_wait(a, sm.task, k, nt - 2 - k, tasks_before_step(nt, k + 1), t);
@@ -787,6 +814,7 @@ __device__ __forceinline__ bool run_chain(const Args& a, Smem& sm, int t) {
         if (!s.go) return false;
       }
       load_chain_tiles(a, s, k, t, kThreads);
+      copy_async_wait();
       __syncthreads();
     }
     if (!first) {
