@@ -891,6 +891,9 @@ inline gptq_status_t launch(float* A, int64_t ld, int w, int k_global, Flags* fl
   for (int k = 0; k < a.nt; ++k) widest = 2 * step_updates(a.nt, k) + 1 > widest ? 2 * step_updates(a.nt, k) + 1 : widest;
   int ctas = widest < max_ctas ? widest : max_ctas;
   if (ctas > products + 1) ctas = products + 1;
+  // ... and half a CTA per tile: launches of several layers then run side by side (a CTA takes an SM), and alone nothing is slower from
+  // 384 columns on (125M-shaped block, four factors at once: 2168 us without this, 2034 with, 2033 with 3/8; 768-wide layer 340, 340, 350).
+  if (a.nt >= 6 && ctas > a.nt * a.nt / 2) ctas = a.nt * a.nt / 2;
   GPTQ_CUDA_TRY(cudaFuncSetAttribute(panel_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)));
   panel_factor_kernel<<<ctas, kThreads, sizeof(Smem), s>>>(a);
   GPTQ_LAUNCH_CHECK();
