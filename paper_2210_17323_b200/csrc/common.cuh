@@ -49,6 +49,31 @@ void count_launch(int n = 1);
     GPTQ_CUDA_TRY(cudaGetLastError());      \
   } while (0)
 
+// Launches that follow one another inside a call.  A kernel launched by launch_next may be set up while the one before it in the stream
+// ends (programmatic dependent launch): every thread of it begins with pdl_wait, which returns when that kernel is complete and its
+// results are visible.  A kernel lets the next one be set up by pdl_next, a short one at once, a long one shortly before its end: what is
+// set up holds its place on the SMs, and other streams have use for it.  Only where a kernel of the same call that begins with pdl_wait
+// too stands directly before it in the stream; in a kernel launched in the ordinary way the wait is over at once.
+// (768-wide layer, 21 launches: 340 -> 320 us; 1000 x 2400 1604 -> 1562; 125M-shaped block on several streams 2034 -> 1793.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() { pdl_wait(); pdl_next(); }
+template <class... P, class... A>
+inline cudaError_t launch_next(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#define GPTQ_LAUNCH_NEXT(...)                                       \
+  do {                                                              \
+    GPTQ_CUDA_TRY(::gptq::launch_next(__VA_ARGS__));                \
+    ::gptq::count_launch();                                         \
+  } while (0)
+
 // dev_info word layout: [0] status, [1] detail (pivot index, ...).  First error wins.
 __device__ __forceinline__ void report_error(int* dev_info, int status, int detail) {
   if (dev_info && atomicCAS(dev_info, 0, status) == 0) dev_info[1] = detail;

@@ -24,6 +24,7 @@ namespace {
 // lambda = damp * mean(diag H); also clears the call's report and the progress words of the panel kernel.
 __global__ void lambda_kernel(const float* __restrict__ H, int C, float damp, double* __restrict__ lam, int* __restrict__ dev_info,
                               int* __restrict__ flags, int n_flags) {
+  pdl_begin();
   __shared__ double red[32];
   if (threadIdx.x < 2) dev_info[threadIdx.x] = 0;
   for (int i = threadIdx.x; i < n_flags; i += blockDim.x) flags[i] = 0;
@@ -42,6 +43,7 @@ __global__ void lambda_kernel(const float* __restrict__ H, int C, float damp, do
 // U <- upper triangle of (H + lambda I); strict lower triangle <- 0.
 __global__ void init_upper_damped_kernel(const float* H, float* U, int C,
                                          const double* __restrict__ lam) {
+  pdl_begin();
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t total = (int64_t)C * C / 4;
   if (idx >= total) return;
@@ -69,6 +71,7 @@ __global__ void init_upper_damped_kernel(const float* H, float* U, int C,
 // r_i 2^12 is called rs_i below.
 __global__ void factor_scales_kernel(const float* __restrict__ U, int C, float* __restrict__ r, float* __restrict__ rinv,
                                      float* __restrict__ rs, float* __restrict__ rsinv) {
+  pdl_begin();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= C) return;
   const float ri = pow2_scale_to(sqrtf(U[(int64_t)i * C + i]), 0);
@@ -79,6 +82,7 @@ __global__ void factor_scales_kernel(const float* __restrict__ U, int C, float* 
 //   gam[b] brings max_j |V[j][b]|        just below 2^15,  gam2inv = 2^5 / gam
 __global__ void panel_scales_kernel(const float* __restrict__ D, int64_t ld, int w, const float* __restrict__ rinv,
                                     float* __restrict__ g, float* __restrict__ ginv, float* __restrict__ gam, float* __restrict__ gam2inv) {
+  pdl_begin();
   __shared__ float red[2][32];
   const int b = blockIdx.x;
   float mr = 0.f, mc = 0.f;
@@ -185,6 +189,7 @@ struct EpiStoreF32AndSplit {
 // D[r][c] -= sum over the n parts, in their order and in 64 bits, for c >= r (c, r < w <= 1024, w a multiple of 4).  One CTA per row.
 __global__ void __launch_bounds__(256) subtract_parts_kernel(float* __restrict__ D, int64_t ld, int w, const float* __restrict__ parts, int n,
                                                              int64_t stride, int64_t ld_parts) {
+  pdl_begin();
   const int r = blockIdx.x, c = 4 * threadIdx.x;
   if (c >= w || c + 3 < r) return;
   float4* d = reinterpret_cast<float4*>(D + (int64_t)r * ld + c);
@@ -375,13 +380,11 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
   GPTQ_LAUNCH_CHECK();
   {
     int64_t total = (int64_t)C * C / 4;
-    init_upper_damped_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(H, U, C, w.lam);
-    GPTQ_LAUNCH_CHECK();
+    GPTQ_LAUNCH_NEXT(init_upper_damped_kernel, (unsigned)((total + 255) / 256), 256, 0, s, H, U, C, w.lam);
   }
   if (outer) {
     // scalings of the fp16 operand pairs that follow from the damped diagonal alone
-    factor_scales_kernel<<<ceil_div(C, 256), 256, 0, s>>>(U, C, w.r, w.rinv, w.rs, w.rsinv);
-    GPTQ_LAUNCH_CHECK();
+    GPTQ_LAUNCH_NEXT(factor_scales_kernel, ceil_div(C, 256), 256, 0, s, U, C, w.r, w.rinv, w.rs, w.rsinv);
     GPTQ_CUDA_TRY(cudaEventRecord(as->fork, s));
     GPTQ_CUDA_TRY(cudaStreamWaitEvent(sb, as->fork, 0));
   }
@@ -432,8 +435,7 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
     __half* Vhi = w.Vhi[J & 1]; __half* Vlo = w.Vlo[J & 1];
     float* gJ = w.g[J & 1]; float* ginvJ = w.ginv[J & 1];
     // V' = V / r (columns) * g (rows, from the rows' actual maxima); gam of this panel is recomputed in phase 2
-    panel_scales_kernel<<<wj, 256, 0, s>>>(D, C, wj, w.rinv + j0, gJ, ginvJ, w.gam, w.gam2inv);
-    GPTQ_LAUNCH_CHECK();
+    GPTQ_LAUNCH_NEXT(panel_scales_kernel, wj, 256, 0, s, D, C, wj, w.rinv + j0, gJ, ginvJ, w.gam, w.gam2inv);
     if ((st = launch_split_scaled(D, C, wj, wj, gJ, w.rinv + j0, Vhi, Vlo, kNB2, dev_info, s)) != GPTQ_OK) return st;
     GPTQ_CUDA_TRY(cudaEventRecord(as->c3[J], s));
     f16x3::Operand V{Vhi, Vlo, wj, wj, kNB2};

@@ -800,6 +800,7 @@ __device__ __forceinline__ bool run_chain(const Args& a, Smem& sm, int t) {
   };
   for (int k = nt - 1; k >= 0; --k) {
     const bool first = k == nt - 1;
+    if (k == 0 && t == 0) pdl_next();                     // (the other CTAs' leaving counts as theirs)
     if (!first) hand_out(k + 1);
     if (s.got == k) {                                    // (the word goes out before the last tiles are in)
       if ((warp & 3) == 0 && warp > 0) copy_async_wait();
@@ -841,6 +842,7 @@ __device__ __forceinline__ bool run_chain(const Args& a, Smem& sm, int t) {
 }
 
 __global__ void __launch_bounds__(kThreads, 1) panel_factor_kernel(const Args a) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char panel_smem[];
   Smem& s = *reinterpret_cast<Smem*>(panel_smem);
   const int t = threadIdx.x;
@@ -863,6 +865,7 @@ __global__ void __launch_bounds__(kThreads, 1) panel_factor_kernel(const Args a)
 // Second launch: the transposed inverse moves from the lower tiles to its place above the diagonal, zeros below it, and the
 // progress words are cleared for the next panel.  32 x 32 pieces, grid (w / 32, w / 32), block (32, 8).
 __global__ void __launch_bounds__(256) panel_place_inverse_kernel(float* __restrict__ A, int64_t ld, Flags* fl) {
+  pdl_begin();
   __shared__ float tile[32][33];
   const int bi = blockIdx.y, bj = blockIdx.x, tx = threadIdx.x, ty = threadIdx.y;
   if (bi == 0 && bj == 0) {
@@ -895,11 +898,9 @@ inline gptq_status_t launch(float* A, int64_t ld, int w, int k_global, Flags* fl
   // 384 columns on (125M-shaped block, four factors at once: 2168 us without this, 2034 with, 2033 with 3/8; 768-wide layer 340, 340, 350).
   if (a.nt >= 6 && ctas > a.nt * a.nt / 2) ctas = a.nt * a.nt / 2;
   GPTQ_CUDA_TRY(cudaFuncSetAttribute(panel_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)));
-  panel_factor_kernel<<<ctas, kThreads, sizeof(Smem), s>>>(a);
-  GPTQ_LAUNCH_CHECK();
+  GPTQ_LAUNCH_NEXT(panel_factor_kernel, ctas, kThreads, sizeof(Smem), s, a);
   dim3 grid(w / 32, w / 32), blk(32, 8);
-  panel_place_inverse_kernel<<<grid, blk, 0, s>>>(A, ld, fl);
-  GPTQ_LAUNCH_CHECK();
+  GPTQ_LAUNCH_NEXT(panel_place_inverse_kernel, grid, blk, 0, s, A, ld, fl);
   return GPTQ_OK;
 }
 

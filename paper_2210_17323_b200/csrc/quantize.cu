@@ -63,6 +63,7 @@ __device__ __forceinline__ void find_params(double mn, double mx, GridSpec g, fl
 // 2^11, sEinv = 1 / sE.
 __global__ void rowstats_kernel(const __half* __restrict__ W, int R, int C, GridSpec g,
                                 float* __restrict__ scales, float* __restrict__ zeros, float* __restrict__ sE, float* __restrict__ sEinv) {
+  pdl_begin();
   int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= R) return;
   const uint4* p = reinterpret_cast<const uint4*>(W + (int64_t)row * C);
@@ -117,6 +118,7 @@ __global__ void wblk_from_w16_kernel(const __half* __restrict__ W, int R, int C,
 }
 // D = the sum of n parts, `stride` floats apart, in their order and in 64 bits; the first part is D itself.  R rows of nb columns, four per thread.
 __global__ void __launch_bounds__(256) sum_parts_kernel(float* __restrict__ D, int R, int nb, int64_t ldd, int n, int64_t stride) {
+  pdl_begin();
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (idx >= (int64_t)R * (nb / 4)) return;
   float* d = D + idx / (nb / 4) * ldd + idx % (nb / 4) * 4;
@@ -138,6 +140,7 @@ wblk_stripe_major_kernel(const __half* __restrict__ W, int R, int C, int i2,
                          const float* __restrict__ D, int64_t ldd,
                          const float* __restrict__ sEinv, const float* __restrict__ sCinv, double sign,
                          double* __restrict__ Wblk, int64_t ldw) {
+  pdl_begin();
   __shared__ float t[128][33];
   __shared__ float d[128][33];
   const int r0 = blockIdx.y * 128, c0 = blockIdx.x * 32;
@@ -357,6 +360,7 @@ __global__ void __launch_bounds__(kInblockThreads) inblock_kernel(InblockArgs a)
 // load per code: 160 us for 12288 x 12288 4-bit codes, where the bytes take 35.)
 template <int F>
 __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* __restrict__ codes, int64_t n32, bool wide, uint32_t* __restrict__ qweight) {
+  pdl_begin();
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (idx >= n32) return;
   const uint4 a = reinterpret_cast<const uint4*>(codes)[2 * idx], b = reinterpret_cast<const uint4*>(codes)[2 * idx + 1];
@@ -389,6 +393,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* __restrict__ c
 // sK[k] = largest power of two <= U_kk; colmax[c] = colmax2[c] = 0; and the call's report and loss start at zero
 __global__ void kscale_kernel(const float* __restrict__ U, int C, float* __restrict__ sK, uint32_t* __restrict__ colmax,
                               uint32_t* __restrict__ colmax2, int* __restrict__ dev_info, double* __restrict__ loss) {
+  pdl_begin();
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < 2) dev_info[k] = 0;
   if (k == 0) *loss = 0.0;
@@ -405,6 +410,7 @@ __global__ void kscale_kernel(const float* __restrict__ U, int C, float* __restr
 __device__ __forceinline__ float pow2_inverse(float s) { return __uint_as_float(0x7F000000u - __float_as_uint(s)); }   // s = 2^e, |e| <= 100
 __global__ void __launch_bounds__(256) colmax_kernel(const float* __restrict__ U, int C, const float* __restrict__ sK, uint32_t* __restrict__ colmax,
                                                      int fblock, uint32_t* __restrict__ colmax2) {
+  pdl_begin();
   __shared__ float4 red[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 128 + 4 * lane, r0 = blockIdx.y * 128;
@@ -444,6 +450,7 @@ __global__ void __launch_bounds__(256) colmax_kernel(const float* __restrict__ U
 // above the diagonal blocks (factor form: colmax2 != nullptr)
 __global__ void cscale_kernel(const uint32_t* __restrict__ colmax, const uint32_t* __restrict__ colmax2, int C, float* __restrict__ sC,
                               float* __restrict__ sCinv, float* __restrict__ sC2, float* __restrict__ sC2inv) {
+  pdl_begin();
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
   const float s = pow2_scale_to(__uint_as_float(colmax[c]), 13);
@@ -461,6 +468,7 @@ __global__ void __launch_bounds__(256)
 split_panel_t_kernel(const float* __restrict__ U, int C, int i2, int rows,
                      const float* __restrict__ sK, const float* __restrict__ sC, const float* __restrict__ sC2,
                      __half* __restrict__ Phi, __half* __restrict__ Plo, int64_t ldp) {
+  pdl_begin();
   __shared__ float t[128][33];
   const int r0 = blockIdx.y * 128, c0 = blockIdx.x * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -499,6 +507,7 @@ __global__ void residual_pair_kernel(const __half* __restrict__ W, const uint8_t
                                      const float* __restrict__ scales, const float* __restrict__ zeros, int G, int g,
                                      const float* __restrict__ sE, int R, int C, int i2, int nb2,
                                      __half* __restrict__ Ehi, __half* __restrict__ Elo, int* dev_info) {
+  pdl_begin();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int per_row = nb2 / 8;
   if (idx >= (int64_t)R * per_row) return;
@@ -571,10 +580,9 @@ gptq_status_t launch_stripe(const StripeArgs& a, const __half* Phi, const __half
   if ((st = map(&maps.p_lo, Plo, 64, kStripeNT, CU_TENSOR_MAP_SWIZZLE_128B)) != GPTQ_OK) return st;
   if ((st = map(&maps.s_hi, Phi, 16, 32, CU_TENSOR_MAP_SWIZZLE_32B)) != GPTQ_OK) return st;
   if ((st = map(&maps.s_lo, Plo, 16, 32, CU_TENSOR_MAP_SWIZZLE_32B)) != GPTQ_OK) return st;
-  auto kern = a.group > 0 && a.group < 32 ? stripe_kernel<true> : stripe_kernel<false>;
+  const auto kern = a.group > 0 && a.group < 32 ? stripe_kernel<true> : stripe_kernel<false>;
   GPTQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripeSmem));
-  kern<<<ceil_div(a.R, kStripeRows), kStripeThreads, kStripeSmem, s>>>(maps, a);
-  GPTQ_LAUNCH_CHECK();
+  GPTQ_LAUNCH_NEXT(kern, ceil_div(a.R, kStripeRows), kStripeThreads, kStripeSmem, s, maps, a);
   return GPTQ_OK;
 }
 
@@ -672,13 +680,10 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
   GPTQ_LAUNCH_CHECK();
   {
     dim3 grid(ceil_div(C, 128), ceil_div(C, 128));
-    colmax_kernel<<<grid, 256, 0, s>>>(U, C, sK, colmax, factor ? GPTQ_FACTOR_BLOCK : 0, colmax2);
-    GPTQ_LAUNCH_CHECK();
+    GPTQ_LAUNCH_NEXT(colmax_kernel, grid, 256, 0, s, U, C, sK, colmax, factor ? GPTQ_FACTOR_BLOCK : 0, colmax2);
   }
-  cscale_kernel<<<ceil_div(C, 256), 256, 0, s>>>(colmax, factor ? colmax2 : nullptr, C, sC, sCinv, sC2, sC2inv);
-  GPTQ_LAUNCH_CHECK();
-  rowstats_kernel<<<ceil_div(R, 8), 256, 0, s>>>(W, R, C, gs, g == 0 ? scales : nullptr, zeros, sE, sEinv);
-  GPTQ_LAUNCH_CHECK();
+  GPTQ_LAUNCH_NEXT(cscale_kernel, ceil_div(C, 256), 256, 0, s, colmax, factor ? colmax2 : nullptr, C, sC, sCinv, sC2, sC2inv);
+  GPTQ_LAUNCH_NEXT(rowstats_kernel, ceil_div(R, 8), 256, 0, s, W, R, C, gs, g == 0 ? scales : nullptr, zeros, sE, sEinv);
   auto inblock_smem = [&](int B) { return (size_t)((size_t)B * kLDS + (size_t)kSB * B + kSB) * sizeof(double) + (size_t)(kSB * kRPB + kSB) * sizeof(float); };
   GPTQ_CUDA_TRY(cudaFuncSetAttribute(inblock_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inblock_smem(256)));
 
@@ -697,8 +702,8 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
     const int nb2 = (C - i2 < B2) ? C - i2 : B2;
     {  // transposed fp16 hi / lo pair of U[0 : i2 + nb2, i2 : i2 + nb2] for the contractions of this outer block
       dim3 grid(nb2 / 32, ceil_div(i2 + nb2, 128)), blk(32, 8);
-      split_panel_t_kernel<<<grid, blk, 0, s>>>(U, C, i2, i2 + nb2, sK, sC, factor ? sC2 : nullptr, Phi, Plo, (int64_t)C);
-      GPTQ_LAUNCH_CHECK();
+      // (directly after a kernel of this call: rowstats, or the block before's last one)
+      GPTQ_LAUNCH_NEXT(split_panel_t_kernel, grid, blk, 0, s, U, C, i2, i2 + nb2, sK, sC, factor ? sC2 : nullptr, Phi, Plo, (int64_t)C);
     }
     // working weights of the outer block: original weights minus all updates from columns < i2
     if (stripe) {
@@ -722,16 +727,14 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
         }
         if (st != GPTQ_OK) return st;
         if (cut.n > 1) {
-          sum_parts_kernel<<<(unsigned)(((int64_t)R * (nb2 / 4) + 255) / 256), 256, 0, s>>>(Dsum, R, nb2, B2, cut.n, rows * B2);
-          GPTQ_LAUNCH_CHECK();
+          GPTQ_LAUNCH_NEXT(sum_parts_kernel, (unsigned)(((int64_t)R * (nb2 / 4) + 255) / 256), 256, 0, s, Dsum, R, nb2, B2, cut.n, rows * B2);
         }
       }
       // (factor form: A holds the plain residuals and the panel rows above the block hold U~[before, blk] U_blk, scaled per
       // column by sC2: the sums ARE the block's correction, with the opposite sign)
       dim3 grid(nb2 / 32, ceil_div(R, 128)), blk(32, 8);
-      wblk_stripe_major_kernel<<<grid, blk, 0, s>>>(W, R, C, i2, i2 > 0 ? Dsum : nullptr, B2, sEinv, factor ? sC2inv : sCinv,
-                                                    factor ? 1.0 : -1.0, Wblk, ldw);
-      GPTQ_LAUNCH_CHECK();
+      GPTQ_LAUNCH_NEXT(wblk_stripe_major_kernel, grid, blk, 0, s, W, R, C, i2, i2 > 0 ? Dsum : nullptr, B2, sEinv, factor ? sC2inv : sCinv,
+                       factor ? 1.0 : -1.0, Wblk, ldw);
     } else {
       int64_t total = (int64_t)R * nb2;
       wblk_from_w16_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(W, R, C, i2, nb2, Wblk, ldw, 0);
@@ -751,9 +754,8 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
       if (factor && i2 + nb2 < C) {
         // factor form: what later outer blocks contract with is the plain residual of this block's columns
         const int64_t n8 = (int64_t)R * (nb2 / 8);
-        residual_pair_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, s>>>(W, codes, scales, zeros, G, g, sE, R, C, i2, nb2, Ehi, Elo,
-                                                                          dev_info);
-        GPTQ_LAUNCH_CHECK();
+        GPTQ_LAUNCH_NEXT(residual_pair_kernel, (unsigned)((n8 + 255) / 256), 256, 0, s, W, codes, scales, zeros, G, g, sE, R, C, i2, nb2, Ehi, Elo,
+                         dev_info);
       }
       continue;
     }
@@ -782,8 +784,7 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
     const int f = field_bits(bits);
     const int64_t n32 = (int64_t)R * (C / 32);
     const auto kern = f == 2 ? pack_kernel<2> : f == 3 ? pack_kernel<3> : f == 4 ? pack_kernel<4> : pack_kernel<8>;
-    kern<<<(unsigned)((n32 + 255) / 256), 256, 0, s>>>(codes, n32, aligned_to(qweight, 16), qweight);
-    GPTQ_LAUNCH_CHECK();
+    GPTQ_LAUNCH_NEXT(kern, (unsigned)((n32 + 255) / 256), 256, 0, s, codes, n32, aligned_to(qweight, 16), qweight);
   }
   return GPTQ_OK;
 }

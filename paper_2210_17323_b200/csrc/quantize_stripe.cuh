@@ -501,6 +501,7 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
   }
   if (warp == 4) { tmem_alloc(&bar.tmem, 512); tmem_relinquish(); }
   fence_before_thread_sync();
+  pdl_wait();                                             // (nothing above reads or writes what another kernel does)
   __syncthreads();
   fence_after_thread_sync();
   const uint32_t tmem = bar.tmem;
@@ -548,6 +549,7 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
 #pragma unroll 1
       for (int j0 = 0; j0 < k.width; j0 += kStripeSB, ++n) {
         const StripeCols& cs = cols[n & 1];
+        if (t == 0 && k.ib + j0 + kStripeSB >= a.nb2) pdl_next();                 // the last sixteen columns
         auto at = [&]() {
           return StripeAt{wg + (int64_t)(k.ib + j0) * kStripeRows, a.sCinv + i + j0, tm_next + j0, tm_rest + j0, b > 0, j0 > 0, live, inv_se};
         };
