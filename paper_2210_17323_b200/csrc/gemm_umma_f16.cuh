@@ -119,7 +119,7 @@ struct Operand {
 // K is longer.
 template <bool kTriLeft, bool kUpperOut, class EpiF>
 gptq_status_t launch(const Operand& A, const Operand& B, int M, int N, EpiF epi, int* dev_info, cudaStream_t stream,
-                     int reserve_sms = 0, const CUtensorMap* out_map = nullptr, int k_item = kSuperK) {
+                     int reserve_sms = 0, const CUtensorMap* out_map = nullptr, int k_item = kSuperK, bool next = false) {
   const int64_t K = A.cols;
   if (M <= 0 || N <= 0 || K <= 0) return GPTQ_OK;
   if (pipe2::is_tile_epilogue<EpiF>::value != (out_map != nullptr)) return GPTQ_ERR_INVALID_ARG;
@@ -138,7 +138,7 @@ gptq_status_t launch(const Operand& A, const Operand& B, int M, int N, EpiF epi,
   const TileItems<kTriLeft, kUpperOut> items{(M + BM - 1) / BM, (N + BN - 1) / BN, (int)((K + BK - 1) / BK), k_item / BK};
   const int n_sc = (items.kb_total + items.sc_kb - 1) / items.sc_kb;
   return pipe2::launch_pipe2<Traits>(maps, (int64_t)items.tiles_m * items.tiles_n * n_sc, items, epi, dev_info, stream,
-                                     reserve_sms);
+                                     reserve_sms, next);
 }
 
 // Scaled sums of one warp's 32 x 32 block, sums * (alpha * sa[row]) * sb[col] (sa, sb optional), into its swizzled 4 KB staging tile.

@@ -209,6 +209,7 @@ __global__ void __launch_bounds__(256) subtract_parts_kernel(float* __restrict__
 __global__ void split_scaled_kernel(const float* __restrict__ src, int64_t ld_src, int rows, int w,
                                     const float* __restrict__ sr, const float* __restrict__ sc,
                                     __half* __restrict__ dhi, __half* __restrict__ dlo, int64_t ld_dst, int* dev_info) {
+  pdl_begin();
   const int q = w / 4;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)rows * q) return;
@@ -231,6 +232,7 @@ __global__ void split_scaled_kernel(const float* __restrict__ src, int64_t ld_sr
 // VT{hi,lo}[c][r] = split(U[j0 + r][j0 + c] * gam[c]) for r, c < w  (transpose of a diagonal block, ld = ldv).
 __global__ void split_diag_t_kernel(const float* __restrict__ U, int C, int j0, const float* __restrict__ gam,
                                     __half* __restrict__ Vhi, __half* __restrict__ Vlo, int ldv) {
+  pdl_begin();
   __shared__ float t[32][33];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   t[threadIdx.y][threadIdx.x] = U[(int64_t)(j0 + r0 + threadIdx.y) * C + j0 + c0 + threadIdx.x];
@@ -415,8 +417,7 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
       st = f16x3::launch<false, true>(A, A, wj, wj, f16x3::EpiTileParts{wj, {wj, 1.f, w.rsinv + j0, w.rsinv + j0}, kNB2, cut.k_item / f16x3::BK},
                                       dev_info, s, 0, &parts, cut.k_item);
       if (st != GPTQ_OK) return st;
-      subtract_parts_kernel<<<wj, 256, 0, s>>>(D, C, wj, w.parts, cut.n, (int64_t)kNB2 * kNB2, kNB2);
-      GPTQ_LAUNCH_CHECK();
+      GPTQ_LAUNCH_NEXT(subtract_parts_kernel, wj, 256, 0, s, D, C, wj, w.parts, cut.n, (int64_t)kNB2 * kNB2, kNB2);
       if (j0 > 0) {
         // B1
         GPTQ_CUDA_TRY(cudaStreamWaitEvent(sb, as->c4[J + 1], 0));
@@ -459,7 +460,7 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
       f16x3::Operand A4{w.TAhi, w.TAlo, kNB2, wj, kNB2};
       st = f16x3::launch<false, false>(A4, V, kNB2, wj,
                                        EpiStoreF32AndSplit{U + o, C, w.Fhi + o, w.Flo + o, C, kNB2, wj, w.rsinv + r1, ginvJ, dev_info},
-                                       dev_info, s);
+                                       dev_info, s, 0, nullptr, f16x3::kSuperK, true);
       if (st != GPTQ_OK) return st;
     }
     GPTQ_CUDA_TRY(cudaEventRecord(as->c4[J], s));
@@ -485,12 +486,12 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
       panel_scales_kernel<<<wj, 256, 0, s>>>(U + (int64_t)j0 * C + j0, C, wj, w.rinv + j0, w.g[0], w.ginv[0], w.gam, w.gam2inv);
       GPTQ_LAUNCH_CHECK();
       dim3 grid(ceil_div(wj, 32), ceil_div(wj, 32)), blk(32, 32);
-      split_diag_t_kernel<<<grid, blk, 0, s>>>(U, C, j0, w.gam, w.VThi, w.VTlo, kNB2);
-      GPTQ_LAUNCH_CHECK();
+      GPTQ_LAUNCH_NEXT(split_diag_t_kernel, grid, blk, 0, s, U, C, j0, w.gam, w.VThi, w.VTlo, kNB2);
       f16x3::Operand A{w.Fhi + j0, w.Flo + j0, j0, wj, C};          // U~[0:j0, J] rs_i
       f16x3::Operand B{w.VThi, w.VTlo, wj, wj, kNB2};               // V_JJ[k][n] gam_n, as [n][k]
       // partial = rs_i gam_n (U~ V)[i][n];  1 / gam_n = gam2inv_n / 32
-      st = f16x3::launch<false, false>(A, B, j0, wj, EpiStoreScaledF32{U + j0, C, j0, wj, w.rsinv, w.gam2inv, 1.f / 32.f}, dev_info, s);
+      st = f16x3::launch<false, false>(A, B, j0, wj, EpiStoreScaledF32{U + j0, C, j0, wj, w.rsinv, w.gam2inv, 1.f / 32.f}, dev_info, s, 0,
+                                       nullptr, f16x3::kSuperK, true);
       if (st != GPTQ_OK) return st;
     }
     return GPTQ_OK;
@@ -508,14 +509,14 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
     panel_scales_kernel<<<wj, 256, 0, s>>>(U + (int64_t)j0 * C + j0, C, wj, w.rinv + j0, w.g[0], w.ginv[0], w.gam, w.gam2inv);
     GPTQ_LAUNCH_CHECK();
     dim3 grid(ceil_div(wj, 32), ceil_div(wj, 32)), blk(32, 32);
-    split_diag_t_kernel<<<grid, blk, 0, s>>>(U, C, j0, w.gam, w.VThi, w.VTlo, kNB2);
-    GPTQ_LAUNCH_CHECK();
+    GPTQ_LAUNCH_NEXT(split_diag_t_kernel, grid, blk, 0, s, U, C, j0, w.gam, w.VThi, w.VTlo, kNB2);
     // TT = V_JJ^T * U~[0:j0, J]^T   (wj x j0), written as a hi / lo pair (single super-chunk: K = wj)
     {
       f16x3::Operand A{w.VThi, w.VTlo, wj, wj, kNB2};
       f16x3::Operand B{w.Fhi + j0, w.Flo + j0, j0, wj, C};
       // partial = gam_j' rs_i T; stored as T r_i gam_j' 2^-5 = partial 2^-17
-      st = f16x3::launch<false, false>(A, B, wj, j0, EpiStoreSplit{w.TThi, w.TTlo, C, wj, j0, 1.f / 131072.f, dev_info}, dev_info, s);
+      st = f16x3::launch<false, false>(A, B, wj, j0, EpiStoreSplit{w.TThi, w.TTlo, C, wj, j0, 1.f / 131072.f, dev_info}, dev_info, s, 0, nullptr,
+                                       f16x3::kSuperK, true);
       if (st != GPTQ_OK) return st;
     }
     GPTQ_CUDA_TRY(cudaMemset2DAsync(U + j0, (size_t)C * 4, 0, (size_t)wj * 4, j0, s));

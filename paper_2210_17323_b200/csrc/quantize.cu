@@ -720,7 +720,7 @@ gptq_status_t quantize_impl(const void* W_fp16, const float* U, int R, int C,
         const f16x3::TileScale plain{R, 1.f, nullptr, nullptr};
         if (cut.n > 0) {
           st = f16x3::launch<false, false>(A, Bop, R, nb2, f16x3::EpiTileParts{nb2, plain, (int)rows, cut.k_item / f16x3::BK}, dev_info, s, 0, &out,
-                                           cut.k_item);
+                                           cut.k_item, true);
         } else {
           GPTQ_CUDA_TRY(cudaMemsetAsync(Dsum, 0, (size_t)R * B2 * sizeof(float), s));
           st = f16x3::launch<false, false>(A, Bop, R, nb2, f16x3::EpiTileAddF32{nb2, plain}, dev_info, s, 0, &out);

@@ -191,6 +191,7 @@ umma_pipe2_kernel(const __grid_constant__ typename Traits::Maps maps, const int 
   __syncthreads();
   cluster_sync();                       // peer's barriers are initialised before anything is sent to them
   fence_after_thread_sync();
+  pdl_wait();                           // (the static form may be launched by launch_next)
   const uint32_t tmem_base = *tmem_slot;
   bool abort = false;
   if constexpr (kDynamic) {
@@ -321,6 +322,7 @@ umma_pipe2_kernel(const __grid_constant__ typename Traits::Maps maps, const int 
       }
     }
   }
+  if constexpr (!kDynamic) { if (warp == 0) pdl_next(); }      // the last operands are in
   fence_before_thread_sync();
   __syncthreads();
   cluster_sync();                       // the peer is done with this CTA's shared memory and barriers
@@ -330,10 +332,10 @@ umma_pipe2_kernel(const __grid_constant__ typename Traits::Maps maps, const int 
 constexpr size_t kBarrierBytes = 512;    // pipeline barriers, TMEM slot and the scheduler ring behind the stages
 
 // Static form: a persistent grid of at most one CTA pair per two SMs (less `reserve_sms`, left free for kernels
-// running beside this one); pair p takes items p, p + pairs, ...
+// running beside this one); pair p takes items p, p + pairs, ...  next: see launch_next.
 template <class Traits, class ItemF, class EpiF>
 gptq_status_t launch_pipe2(const typename Traits::Maps& maps, int64_t n_items, ItemF itemf, EpiF epi, int* dev_info,
-                           cudaStream_t stream, int reserve_sms = 0) {
+                           cudaStream_t stream, int reserve_sms = 0, bool next = false) {
   if (n_items <= 0) return GPTQ_OK;
   if (n_items > 0x7FFFFFFF) return GPTQ_ERR_UNSUPPORTED;
   constexpr size_t smem = (size_t)Traits::STAGES * Traits::STAGE_BYTES + epi_smem_of<Traits>::value + 1024 + kBarrierBytes;
@@ -342,8 +344,12 @@ gptq_status_t launch_pipe2(const typename Traits::Maps& maps, int64_t n_items, I
   const int pairs = (int)(n_items < pairs_max ? n_items : pairs_max);
   auto kern = umma_pipe2_kernel<Traits, ItemF, EpiF, false>;
   GPTQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<2 * pairs, threads_of(false), smem, stream>>>(maps, (int)n_items, itemf, epi, dev_info);
-  GPTQ_LAUNCH_CHECK();
+  if (next) {
+    GPTQ_LAUNCH_NEXT(kern, 2 * pairs, threads_of(false), smem, stream, maps, (int)n_items, itemf, epi, dev_info);
+  } else {
+    kern<<<2 * pairs, threads_of(false), smem, stream>>>(maps, (int)n_items, itemf, epi, dev_info);
+    GPTQ_LAUNCH_CHECK();
+  }
   return GPTQ_OK;
 }
 
