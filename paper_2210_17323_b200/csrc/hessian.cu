@@ -51,6 +51,7 @@ struct AddTwiceUpper {
 constexpr int kMirrorTile = 64;
 __global__ void __launch_bounds__(256) mirror_upper_to_lower_kernel(float* __restrict__ H, int C) {
   __shared__ float t[kMirrorTile][kMirrorTile + 1];
+  pdl_wait();
   // linear index -> (bi <= bj): column bj holds the tiles bj (bj + 1) / 2 ...
   const int idx = blockIdx.x;
   int bj = (int)((sqrtf(8.f * (float)idx + 1.f) - 1.f) * 0.5f);
@@ -89,8 +90,12 @@ __global__ void __launch_bounds__(256) mirror_upper_to_lower_kernel(float* __res
 
 }  // namespace
 
-cudaError_t launch_mirror_upper_to_lower(float* H, int C, cudaStream_t stream) {
+cudaError_t launch_mirror_upper_to_lower(float* H, int C, cudaStream_t stream, bool next) {
   const int64_t n = ceil_div(C, kMirrorTile), tiles = n * (n + 1) / 2;
+  if (next) {
+    count_launch();
+    return launch_next(mirror_upper_to_lower_kernel, (unsigned)tiles, 256, 0, stream, H, C);
+  }
   mirror_upper_to_lower_kernel<<<(unsigned)tiles, 256, 0, stream>>>(H, C);
   count_launch();
   return cudaGetLastError();
@@ -109,7 +114,7 @@ static gptq_status_t hessian_simt(float* H, const __nv_bfloat16* X, int64_t n_to
     GPTQ_CUDA_TRY(launch_gemm_simt(C, C, nz, XtAsA{x, C}, XtAsB{x, C}, UpperTilesSplitK{nt},
                                    AddTwiceUpper{H, C}, stream));
   }
-  if (mirror) GPTQ_CUDA_TRY(launch_mirror_upper_to_lower(H, C, stream));
+  if (mirror) GPTQ_CUDA_TRY(launch_mirror_upper_to_lower(H, C, stream, false));
   return GPTQ_OK;
 }
 
@@ -148,6 +153,6 @@ extern "C" gptq_status_t gptq_hessian_accumulate_upper(float* H, const void* X_b
 extern "C" gptq_status_t gptq_hessian_symmetrize(float* H, int C, void* stream) {
   using namespace gptq;
   if (!H || C <= 0 || C % 32 != 0 || !aligned_to(H, 16)) return GPTQ_ERR_INVALID_ARG;
-  GPTQ_CUDA_TRY(launch_mirror_upper_to_lower(H, C, static_cast<cudaStream_t>(stream)));
+  GPTQ_CUDA_TRY(launch_mirror_upper_to_lower(H, C, static_cast<cudaStream_t>(stream), false));
   return GPTQ_OK;
 }

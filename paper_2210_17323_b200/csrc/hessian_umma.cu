@@ -309,7 +309,7 @@ gptq_status_t hessian_umma(float* H, const __nv_bfloat16* X, int64_t n_tokens, i
                                        dev_info, stream);
   }
   if (st != GPTQ_OK) return st;
-  if (mirror) GPTQ_CUDA_TRY(launch_mirror_upper_to_lower(H, C, stream));
+  if (mirror) GPTQ_CUDA_TRY(launch_mirror_upper_to_lower(H, C, stream, true));
   return GPTQ_OK;
 }
 

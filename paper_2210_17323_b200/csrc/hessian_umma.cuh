@@ -8,5 +8,6 @@ bool hessian_umma_supported(int C, int64_t n_tokens);
 gptq_status_t hessian_umma(float* H, const __nv_bfloat16* X, int64_t n_tokens, int C, int* dev_info,
                            cudaStream_t stream, bool mirror = true);
 
-cudaError_t launch_mirror_upper_to_lower(float* H, int C, cudaStream_t stream);
+// next: directly after a kernel of the same call, see launch_next
+cudaError_t launch_mirror_upper_to_lower(float* H, int C, cudaStream_t stream, bool next);
 }  // namespace gptq

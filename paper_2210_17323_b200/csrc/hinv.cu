@@ -102,6 +102,7 @@ __global__ void panel_scales_kernel(const float* __restrict__ D, int64_t ld, int
 // u[i] brings the diagonal entry of row i of the inverse, U_ii / r_i, to about 2^9;  uinv = 1 / u
 __global__ void inverse_row_scales_kernel(const float* __restrict__ U, int C, const float* __restrict__ rinv,
                                           float* __restrict__ u, float* __restrict__ uinv) {
+  pdl_next();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= C) return;
   const float ui = pow2_scale_to(fabsf(U[(int64_t)i * C + i]) * rinv[i], 9);
@@ -339,12 +340,17 @@ gptq_status_t get_async(HinvAsync** out) {
   return GPTQ_OK;
 }
 
+// next: directly after a kernel of the same call, see launch_next
 gptq_status_t launch_split_scaled(const float* src, int64_t ld_src, int rows, int w, const float* sr, const float* sc,
-                                  __half* dhi, __half* dlo, int64_t ld_dst, int* dev_info, cudaStream_t s) {
+                                  __half* dhi, __half* dlo, int64_t ld_dst, int* dev_info, cudaStream_t s, bool next) {
   if (rows <= 0 || w <= 0) return GPTQ_OK;
   const int64_t total = (int64_t)rows * (w / 4);
-  split_scaled_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(src, ld_src, rows, w, sr, sc, dhi, dlo, ld_dst, dev_info);
-  GPTQ_LAUNCH_CHECK();
+  if (next) {
+    GPTQ_LAUNCH_NEXT(split_scaled_kernel, (unsigned)((total + 255) / 256), 256, 0, s, src, ld_src, rows, w, sr, sc, dhi, dlo, ld_dst, dev_info);
+  } else {
+    split_scaled_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(src, ld_src, rows, w, sr, sc, dhi, dlo, ld_dst, dev_info);
+    GPTQ_LAUNCH_CHECK();
+  }
   return GPTQ_OK;
 }
 }  // namespace
@@ -437,14 +443,14 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
     float* gJ = w.g[J & 1]; float* ginvJ = w.ginv[J & 1];
     // V' = V / r (columns) * g (rows, from the rows' actual maxima); gam of this panel is recomputed in phase 2
     GPTQ_LAUNCH_NEXT(panel_scales_kernel, wj, 256, 0, s, D, C, wj, w.rinv + j0, gJ, ginvJ, w.gam, w.gam2inv);
-    if ((st = launch_split_scaled(D, C, wj, wj, gJ, w.rinv + j0, Vhi, Vlo, kNB2, dev_info, s)) != GPTQ_OK) return st;
+    if ((st = launch_split_scaled(D, C, wj, wj, gJ, w.rinv + j0, Vhi, Vlo, kNB2, dev_info, s, true)) != GPTQ_OK) return st;
     GPTQ_CUDA_TRY(cudaEventRecord(as->c3[J], s));
     f16x3::Operand V{Vhi, Vlo, wj, wj, kNB2};
     const int r1 = j0 - kNB2;                       // first row of row block J-1
     // B2 (rows above row block J-1)
     if (r1 > 0) {
       GPTQ_CUDA_TRY(cudaStreamWaitEvent(sb, as->c3[J], 0));
-      if ((st = launch_split_scaled(U + j0, C, r1, wj, w.rs, w.r + j0, w.TThi, w.TTlo, kNB2, dev_info, sb)) != GPTQ_OK) return st;
+      if ((st = launch_split_scaled(U + j0, C, r1, wj, w.rs, w.r + j0, w.TThi, w.TTlo, kNB2, dev_info, sb, false)) != GPTQ_OK) return st;
       f16x3::Operand A2{w.TThi, w.TTlo, r1, wj, kNB2};
       st = f16x3::launch<false, false>(A2, V, r1, wj,
                                        EpiStoreF32AndSplit{U + j0, C, w.Fhi + j0, w.Flo + j0, C, r1, wj, w.rsinv, ginvJ, dev_info},
@@ -456,7 +462,7 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
     if (K > 0) GPTQ_CUDA_TRY(cudaStreamWaitEvent(s, as->b1[J], 0));
     {
       const int64_t o = (int64_t)r1 * C + j0;
-      if ((st = launch_split_scaled(U + o, C, kNB2, wj, w.rs + r1, w.r + j0, w.TAhi, w.TAlo, kNB2, dev_info, s)) != GPTQ_OK) return st;
+      if ((st = launch_split_scaled(U + o, C, kNB2, wj, w.rs + r1, w.r + j0, w.TAhi, w.TAlo, kNB2, dev_info, s, false)) != GPTQ_OK) return st;
       f16x3::Operand A4{w.TAhi, w.TAlo, kNB2, wj, kNB2};
       st = f16x3::launch<false, false>(A4, V, kNB2, wj,
                                        EpiStoreF32AndSplit{U + o, C, w.Fhi + o, w.Flo + o, C, kNB2, wj, w.rsinv + r1, ginvJ, dev_info},
@@ -502,12 +508,11 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
   for (int J = 1; J < n_outer; ++J) {
     const int j0 = J * kNB2, wj = (C - j0 < kNB2) ? C - j0 : kNB2, rows_p = j0 + wj;
     if (J == 1) {                                   // row scales of the inverse; split copy of its first panel
-      inverse_row_scales_kernel<<<ceil_div(C, 256), 256, 0, s>>>(U, C, w.rinv, w.u, w.uinv);
+      inverse_row_scales_kernel<<<ceil_div(C, 256), 256, 0, s>>>(U, C, w.rinv, w.u, w.uinv);     // (behind an event wait)
       GPTQ_LAUNCH_CHECK();
-      if ((st = launch_split_scaled(U, C, kNB2, kNB2, w.u, w.rinv, w.Fhi, w.Flo, C, dev_info, s)) != GPTQ_OK) return st;
+      if ((st = launch_split_scaled(U, C, kNB2, kNB2, w.u, w.rinv, w.Fhi, w.Flo, C, dev_info, s, true)) != GPTQ_OK) return st;
     }
-    panel_scales_kernel<<<wj, 256, 0, s>>>(U + (int64_t)j0 * C + j0, C, wj, w.rinv + j0, w.g[0], w.ginv[0], w.gam, w.gam2inv);
-    GPTQ_LAUNCH_CHECK();
+    GPTQ_LAUNCH_NEXT(panel_scales_kernel, wj, 256, 0, s, U + (int64_t)j0 * C + j0, C, wj, w.rinv + j0, w.g[0], w.ginv[0], w.gam, w.gam2inv);
     dim3 grid(ceil_div(wj, 32), ceil_div(wj, 32)), blk(32, 32);
     GPTQ_LAUNCH_NEXT(split_diag_t_kernel, grid, blk, 0, s, U, C, j0, w.gam, w.VThi, w.VTlo, kNB2);
     // TT = V_JJ^T * U~[0:j0, J]^T   (wj x j0), written as a hi / lo pair (single super-chunk: K = wj)
@@ -532,7 +537,7 @@ gptq_status_t prepare_impl(const float* H, float damp, int C, float* U, void* ws
       if (st != GPTQ_OK) return st;
     }
     if (J + 1 < n_outer) {
-      if ((st = launch_split_scaled(U + j0, C, rows_p, wj, w.u, w.rinv + j0, w.Fhi + j0, w.Flo + j0, C, dev_info, s)) != GPTQ_OK) return st;
+      if ((st = launch_split_scaled(U + j0, C, rows_p, wj, w.u, w.rinv + j0, w.Fhi + j0, w.Flo + j0, C, dev_info, s, true)) != GPTQ_OK) return st;
     }
   }
   return GPTQ_OK;

@@ -22,7 +22,7 @@
 // in registers; T T^T and the inverse, which nothing else waits for, follow at their own pace.
 // Measured, columns of one call: as separate launches 768 / 1024 0.94 / 1.29 ms; this list with a chain of eight warps that met at a barrier
 // twice every eight columns, roots on it, 0.189 / 0.247 (30,600 cycles a step); this form 0.141 / 0.182 (20,000, of which 17,500 the chain's
-// own and the rest waiting for products).
+// own and the rest waiting for products; 0.135 / 0.176 with the launches around it set up early).
 #pragma once
 
 namespace gptq {
