@@ -237,6 +237,46 @@ def test_panel_factorisation_at_tile_edges(B, C):
             assert ((U - ref).norm(dim=1) / ref.norm(dim=1)).max() <= 1e-4
 
 
+@pytest.mark.parametrize("R,C", [(96, 768), (96, 1280), (300, 2080)])
+@pytest.mark.parametrize("factor", [False, True])
+def test_dependent_launches_give_the_same_in_a_graph_and_one_after_the_other(B, R, C, factor):
+    """Kernels of a call are set up while the one before them ends.  The same call three times without a pause, and captured into a graph and
+    replayed twice, over buffers that hold something else each time, gives the same factor, codes and grids bit for bit."""
+    r = np.random.default_rng(R + C)
+    X = r.standard_normal((2 * C, C)) * np.exp(r.standard_normal(C))
+    H = torch.from_numpy((2 * X.T @ X).astype(np.float32)).cuda()
+    W = torch.from_numpy((0.02 * r.standard_normal((R, C))).astype(np.float16)).cuda()
+    ws = torch.empty(max(B.gptq_prepare_hinv_workspace_bytes(C), B.gptq_quantize_workspace_bytes(R, C, 4, 0, 128)), dtype=torch.uint8, device="cuda")
+    U = torch.empty((C, C), device="cuda")
+
+    def solve():
+        _, info = B.gptq_prepare_hinv(H, 0.01, U=U, ws=ws, factor=factor)
+        out = B.gptq_quantize_layer(W, U, 4, 0, False, 128, ws=ws, factor=factor)
+        return U.clone(), out["qweight"], out["scales"], out["zeros"], info, out["dev_info"]
+
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        ref = solve()
+        torch.cuda.synchronize()
+        again = [solve() for _ in range(3)]
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=side):
+            captured = solve()
+    for _ in range(2):
+        U.fill_(float("nan"))
+        ws.fill_(0xA5)
+        for t in captured:
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        again.append(tuple(t.clone() for t in captured))
+    assert ref[4].tolist() == [0, 0] and ref[5].tolist() == [0, 0]
+    for got in again:
+        assert all(torch.equal(a, b) for a, b in zip(ref, got))
+
+
 @pytest.mark.parametrize("C", [64, 128, 160])
 @pytest.mark.parametrize("exponent", [0, 20, 55])
 def test_panel_pivots_over_the_range(B, C, exponent):
