@@ -580,7 +580,7 @@ gptq_status_t launch_stripe(const StripeArgs& a, const __half* Phi, const __half
   if ((st = map(&maps.p_lo, Plo, 64, kStripeNT, CU_TENSOR_MAP_SWIZZLE_128B)) != GPTQ_OK) return st;
   if ((st = map(&maps.s_hi, Phi, 16, 32, CU_TENSOR_MAP_SWIZZLE_32B)) != GPTQ_OK) return st;
   if ((st = map(&maps.s_lo, Plo, 16, 32, CU_TENSOR_MAP_SWIZZLE_32B)) != GPTQ_OK) return st;
-  const auto kern = a.group > 0 && a.group < 32 ? stripe_kernel<true> : stripe_kernel<false>;
+  const auto kern = a.group <= 0 || a.group >= 128 ? stripe_kernel<kWide> : a.group < 32 ? stripe_kernel<kSmall> : stripe_kernel<kNarrow>;
   GPTQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripeSmem));
   GPTQ_LAUNCH_NEXT(kern, ceil_div(a.R, kStripeRows), kStripeThreads, kStripeSmem, s, maps, a);
   return GPTQ_OK;

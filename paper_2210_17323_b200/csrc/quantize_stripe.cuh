@@ -168,11 +168,35 @@ struct StripeAt {
 // in TMEM (Section 5, grouping).  Out of line, like everything that not every sub-block runs: the loop of the row threads
 // is a few thousand instructions long, and cold code between them costs instruction fetch (136 instead of 95 cycles a
 // column in a small model of the loop).
+// Two forms: stripe_scan starts from memory; stripe_scan_rest goes on behind the first sixteen columns, whose minimum and maximum the caller
+// has from its registers, and is a third shorter for groups of 32 (1000 x 2400, 64-column blocks: 858 -> 795 us; groups of 64, 2048 x 2048
+// 604 -> 590).  For wider groups it saves less than the weights that the caller then holds across the call cost (groups of 128, 4096 x 1024
+// 273.5 -> 276.5 us), so those keep the first, in an instance of the kernel of their own with the per-row grids (224.8 -> 228.1 there).
 __device__ __noinline__ float2 stripe_scan(const StripeAt& at, int width, int pending, GridSpec gs) {
   double mn = INFINITY, mx = -INFINITY, x[kStripeSB], y[kStripeSB];
   stripe_fetch(at.wcol, at.live, x);
 #pragma unroll 1
   for (int c = 0; c < width; c += kStripeSB) {
+    if (c + kStripeSB < width) stripe_fetch(at.wcol + (int64_t)(c + kStripeSB) * kStripeRows, at.live, y);
+    if (c < pending) {
+      float sc[kStripeSB];
+#pragma unroll
+      for (int m = 0; m < kStripeSB; ++m) sc[m] = __ldg(at.sCinv + c + m);
+      if (at.has_next) stripe_subtract(at.next + c, sc, at.inv_se, x);
+      if (at.has_rest) stripe_subtract(at.rest + c, sc, at.inv_se, x);
+    }
+#pragma unroll
+    for (int m = 0; m < kStripeSB; ++m) { mn = x[m] < mn ? x[m] : mn; mx = x[m] > mx ? x[m] : mx; x[m] = y[m]; }
+  }
+  float2 r;
+  find_params(mn, mx, gs, r.x, r.y);
+  return r;
+}
+__device__ __noinline__ float2 stripe_scan_rest(const StripeAt& at, int width, int pending, GridSpec gs, double mn, double mx) {
+  double x[kStripeSB], y[kStripeSB];
+  stripe_fetch(at.wcol + (int64_t)kStripeSB * kStripeRows, at.live, x);
+#pragma unroll 1
+  for (int c = kStripeSB; c < width; c += kStripeSB) {
     if (c + kStripeSB < width) stripe_fetch(at.wcol + (int64_t)(c + kStripeSB) * kStripeRows, at.live, y);
     if (c < pending) {
       float sc[kStripeSB];
@@ -470,12 +494,14 @@ __device__ __forceinline__ void stripe_drain_far(const StripeArgs& a, StripeBars
   }
 }
 
-// kSmallGroups: groups of 4, 8 or 16 columns (their grids are taken inside the column loop; the tests for that cost every
-// other grid 14 cycles a column).
-template <bool kSmallGroups>
+// kGroups: kSmall groups of 4, 8 or 16 columns (their grids are taken inside the column loop; the tests for that cost every
+// other grid 14 cycles a column), kNarrow groups of 32 to 127 (see stripe_scan_rest), kWide the rest and per-row grids.
+enum StripeGroupWidth { kWide, kSmall, kNarrow };
+template <int kGroups>
 __global__ void __launch_bounds__(kStripeThreads, 1)
 stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
   using namespace umma;
+  constexpr bool kSmallGroups = kGroups == kSmall;
   extern __shared__ uint8_t smem_raw[];
   // An offset onto the array, not a rounded address: that would lose the address space, and every read of U in the column loop would
   // be a generic load (4096 rows x 1024 columns, 4-bit: 226 us with those, 198 with shared loads; groups of 128: 287, 249).
@@ -556,7 +582,12 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
         stripe_wait(&bar.cols_full[n & 1], n >> 1, ok, a.dev_info, 36);
         if (n > 0) stripe_wait(&bar.near_done, n - 1, ok, a.dev_info, 37);
         fence_after_thread_sync();
-        if (g >= 32 && ((i + j0) % g) == 0) {              // a group starts (wider than the block: only at j0 = 0)
+        const bool starts = !kSmallGroups && g >= 32 && ((i + j0) % g) == 0;     // a group starts (wider than the block: only at j0 = 0)
+        auto set_grid = [&](float2 sz) {
+          grid.set(sz);
+          if (live) { a.scales[(int64_t)row * G + (i + j0) / g] = sz.x; a.zeros[(int64_t)row * G + (i + j0) / g] = sz.y; }
+        };
+        if (starts) {
           if (g > a.B) {
             const int q = min(b - 1, (a.nb2 + a.B - 1) / a.B - 3);        // the last block before this one with far pushes
             if (q >= 0) stripe_wait(&bar.all_ready[q & 1], q >> 1, ok, a.dev_info, 42);
@@ -564,9 +595,7 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
             stripe_wait(&bar.rest_done, n - 1, ok, a.dev_info, 43);
             fence_after_thread_sync();
           }
-          const float2 sz = stripe_scan(at(), g, k.width - j0, a.grid);
-          grid.set(sz);
-          if (live) { a.scales[(int64_t)row * G + (i + j0) / g] = sz.x; a.zeros[(int64_t)row * G + (i + j0) / g] = sz.y; }
+          if (kGroups != kNarrow) set_grid(stripe_scan(at(), g, k.width - j0, a.grid));
         }
         double w[kStripeSB];
 #pragma unroll
@@ -585,6 +614,12 @@ stripe_kernel(const __grid_constant__ StripeMaps maps, const StripeArgs a) {
           const int col = k.ib + j0 + kStripeSB;
           if (j0 + kStripeSB == k.width && b >= 1 && col < a.nb2) stripe_wait(&bar.next_ready[(b - 1) & 1], (b - 1) >> 1, ok, a.dev_info, 44);
           if (col < a.nb2) stripe_fetch(wg + (int64_t)col * kStripeRows, live, ahead);
+        }
+        if (kGroups == kNarrow && starts) {
+          double mn = w[0], mx = w[0];
+#pragma unroll
+          for (int m = 1; m < kStripeSB; ++m) { mn = w[m] < mn ? w[m] : mn; mx = w[m] > mx ? w[m] : mx; }
+          set_grid(stripe_scan_rest(at(), g, k.width - j0, a.grid, mn, mx));
         }
         StripeGroups sg{g, small_group_starts, a.grid, a.scales + (int64_t)row * G + (i + j0) / (g > 0 ? g : 1),
                         a.zeros + (int64_t)row * G + (i + j0) / (g > 0 ? g : 1), live};

@@ -189,6 +189,24 @@ def test_row_stripe_block_edges(B, R, C, bits, group, block):
                            W16, bits, C, H)
 
 
+@pytest.mark.parametrize("R,C,bits,group,block", [
+    (1, 256, 8, 32, 128),       # one row; four groups inside a block
+    (130, 384, 3, 32, 32),      # a group is a block
+    (129, 1536, 3, 64, 32),     # wider than the block: its second half is in memory only, with two outer blocks
+    (64, 1152, 4, 96, 96),      # the widest but one of this instance, with blocks that do not nest with 128
+    (40, 1440, 2, 96, 32),      # three blocks a group
+    (33, 1088, 3, 64, 64),      # a last outer block of 64 columns
+])
+def test_grids_of_narrow_groups(B, R, C, bits, group, block):
+    """Groups of 32 to 127 columns take the first sixteen columns' share of their grid from the weights in registers; against the oracle."""
+    L = _layer(R, C, 2 * C + 64, cfg=7)
+    W16 = L.w()
+    H = O.hessian_accumulate(np.zeros((C, C)), L.x_bits())
+    U32 = O.cholesky_inverse_upper(O.dampen(H, 0.01)[0]).astype(np.float32)
+    check_quantize_outputs(_run_quant(B, W16, U32, bits, group, False, block), O.quantize_layer(W16, U32.astype(np.float64), bits, group, False, block),
+                           W16, bits, C, H)
+
+
 @pytest.mark.parametrize("bits,group,block,rms,mean", [(2, 32, 32, 1e-7, 6e-8), (3, 8, 32, 4.2e-8, 6.5e-9), (3, 64, 64, 5.2e-8, 2.3e-8)])
 def test_sums_run_over_no_more_columns_than_the_callers_block(B, bits, group, block, rms, mean):
     """The weights that a group's grid is taken from, against a 64-bit replay of the call's own codes and grids.  A tensor-core sum
